@@ -10,7 +10,7 @@
 //
 // The volume term couples only the points of one element.  So a CTA can take
 // a tile of elements through all 5 * nsteps stages with q and dq of its
-// points in registers: q is read from and written to HBM once, and there is
+// points on chip: q is read from and written to HBM once, and there is
 // no grid-wide synchronisation.  The tile's geometry (56 KB in FP64 for one
 // Nq = 8 element) is re-read every stage; after the first stage it comes from
 // L2.  Each stage
@@ -34,7 +34,7 @@ namespace {
 
 // TR: the tiles' tracer forms, for batches that hold instances with tracers.
 template <bool MIXED, bool TR = false>
-__global__ void __launch_bounds__(kThreads, tile_ctas_per_sm<MIXED>())
+__global__ void __launch_bounds__(kThreads, (tile_ctas_per_sm<MIXED, TR>()))
 batch_lsrk_kernel(const BatchInstance *__restrict__ inst, const BatchItem *__restrict__ items,
                   int num_items, int *counter, LsrkCoef co, int nsteps, double dt) {
     extern __shared__ __align__(16) double smem_d[];
@@ -58,13 +58,13 @@ batch_lsrk_kernel(const BatchInstance *__restrict__ inst, const BatchItem *__res
         __syncthreads();
         const int ns = sI.nsteps > 0 ? sI.nsteps : nsteps;
         switch (item.nq) {
-            case 2: run_tile<2, MIXED, TR>(sI, item.e0, item.count, sco, ns, dt, smem_d); break;
-            case 3: run_tile<3, MIXED, TR>(sI, item.e0, item.count, sco, ns, dt, smem_d); break;
-            case 4: run_tile<4, MIXED, TR>(sI, item.e0, item.count, sco, ns, dt, smem_d); break;
-            case 5: run_tile<5, MIXED, TR>(sI, item.e0, item.count, sco, ns, dt, smem_d); break;
-            case 6: run_tile<6, MIXED, TR>(sI, item.e0, item.count, sco, ns, dt, smem_d); break;
-            case 7: run_tile<7, MIXED, TR>(sI, item.e0, item.count, sco, ns, dt, smem_d); break;
-            case 8: run_tile<8, MIXED, TR>(sI, item.e0, item.count, sco, ns, dt, smem_d); break;
+            case 2: run_tile_either_way<2, MIXED, TR>(sI, item.e0, item.count, sco, ns, dt, smem_d); break;
+            case 3: run_tile_either_way<3, MIXED, TR>(sI, item.e0, item.count, sco, ns, dt, smem_d); break;
+            case 4: run_tile_either_way<4, MIXED, TR>(sI, item.e0, item.count, sco, ns, dt, smem_d); break;
+            case 5: run_tile_either_way<5, MIXED, TR>(sI, item.e0, item.count, sco, ns, dt, smem_d); break;
+            case 6: run_tile_either_way<6, MIXED, TR>(sI, item.e0, item.count, sco, ns, dt, smem_d); break;
+            case 7: run_tile_either_way<7, MIXED, TR>(sI, item.e0, item.count, sco, ns, dt, smem_d); break;
+            case 8: run_tile_either_way<8, MIXED, TR>(sI, item.e0, item.count, sco, ns, dt, smem_d); break;
             default: break;
         }
         __syncthreads();   // sI and s_item are rewritten by the next claim
@@ -210,7 +210,8 @@ cudaError_t prepare_batch_lsrk() {
                                 kTcSmemBytes);
 }
 
-int batch_max_ctas_per_sm(bool mixed) { return mixed ? 2 : tile_ctas_per_sm<false>(); }
+// FP64 has one grid (two CTAs per SM, one in the tracer form): its setting is 1.
+int batch_max_ctas_per_sm(bool mixed) { return mixed ? 2 : 1; }
 
 cudaError_t launch_batch_lsrk(bool mixed, const BatchInstance *inst, const BatchItem *items,
                               int num_items, int *counter, const LsrkCoef &co, int nsteps,
@@ -223,7 +224,7 @@ cudaError_t launch_batch_lsrk(bool mixed, const BatchInstance *inst, const Batch
         batch_lsrk_kernel<true, true><<<num_sms * k, kThreads, tile_smem_bytes<true, true>(), s>>>(
             inst, items, num_items, counter, co, nsteps, dt);
     else if (tracers)
-        batch_lsrk_kernel<false, true><<<num_sms * k, kThreads, tile_smem_bytes<false, true>(), s>>>(
+        batch_lsrk_kernel<false, true><<<num_sms * tile_ctas_per_sm<false, true>(), kThreads, tile_smem_bytes<false, true>(), s>>>(
             inst, items, num_items, counter, co, nsteps, dt);
     else if (mixed && (tc_mask != 0 || tmem_state))
         batch_lsrk_tc_kernel<<<num_sms * k, kThreads, kTcSmemBytes, s>>>(
@@ -232,7 +233,7 @@ cudaError_t launch_batch_lsrk(bool mixed, const BatchInstance *inst, const Batch
         batch_lsrk_kernel<true><<<num_sms * k, kThreads, tile_smem_bytes<true>(), s>>>(
             inst, items, num_items, counter, co, nsteps, dt);
     else
-        batch_lsrk_kernel<false><<<num_sms * k, kThreads, tile_smem_bytes<false>(), s>>>(
+        batch_lsrk_kernel<false><<<num_sms * tile_ctas_per_sm<false>(), kThreads, tile_smem_bytes<false>(), s>>>(
             inst, items, num_items, counter, co, nsteps, dt);
     return cudaGetLastError();
 }

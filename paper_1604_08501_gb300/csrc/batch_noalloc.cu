@@ -46,7 +46,7 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
 // TR: the tiles' tracer forms, for a call that holds an instance with tracers.
 template <bool MIXED, bool TR>
-__global__ void __launch_bounds__(kThreads, tile_ctas_per_sm<MIXED>())
+__global__ void __launch_bounds__(kThreads, (tile_ctas_per_sm<MIXED, TR>()))
 batch_lsrk_noalloc_kernel(unsigned char *scratch, LsrkCoef co, int nsteps, double dt) {
     int *counter = reinterpret_cast<int *>(scratch);
     const NoallocTable *tab = reinterpret_cast<const NoallocTable *>(scratch + kCounterBytes);
@@ -77,13 +77,13 @@ batch_lsrk_noalloc_kernel(unsigned char *scratch, LsrkCoef co, int nsteps, doubl
         const int64_t count = ne - e0 < tile ? ne - e0 : tile;
         const int ns = sI.nsteps > 0 ? sI.nsteps : nsteps;
         switch (nq) {
-            case 2: run_tile<2, MIXED, TR>(sI, e0, count, sco, ns, dt, smem_d); break;
-            case 3: run_tile<3, MIXED, TR>(sI, e0, count, sco, ns, dt, smem_d); break;
-            case 4: run_tile<4, MIXED, TR>(sI, e0, count, sco, ns, dt, smem_d); break;
-            case 5: run_tile<5, MIXED, TR>(sI, e0, count, sco, ns, dt, smem_d); break;
-            case 6: run_tile<6, MIXED, TR>(sI, e0, count, sco, ns, dt, smem_d); break;
-            case 7: run_tile<7, MIXED, TR>(sI, e0, count, sco, ns, dt, smem_d); break;
-            case 8: run_tile<8, MIXED, TR>(sI, e0, count, sco, ns, dt, smem_d); break;
+            case 2: run_tile_either_way<2, MIXED, TR>(sI, e0, count, sco, ns, dt, smem_d); break;
+            case 3: run_tile_either_way<3, MIXED, TR>(sI, e0, count, sco, ns, dt, smem_d); break;
+            case 4: run_tile_either_way<4, MIXED, TR>(sI, e0, count, sco, ns, dt, smem_d); break;
+            case 5: run_tile_either_way<5, MIXED, TR>(sI, e0, count, sco, ns, dt, smem_d); break;
+            case 6: run_tile_either_way<6, MIXED, TR>(sI, e0, count, sco, ns, dt, smem_d); break;
+            case 7: run_tile_either_way<7, MIXED, TR>(sI, e0, count, sco, ns, dt, smem_d); break;
+            case 8: run_tile_either_way<8, MIXED, TR>(sI, e0, count, sco, ns, dt, smem_d); break;
             default: break;
         }
         __syncthreads();   // sI and s_item are rewritten by the next claim
@@ -205,7 +205,7 @@ extern "C" int numa_batch_advance_noalloc(const numa_vol *const *handles, void *
         cudaMemsetAsync(ds.scratch, 0, sizeof(int), s) != cudaSuccess)
         return NUMA_ECUDA;
     const int g_mixed = ds.num_sms * tile_ctas_per_sm<true>();
-    const int g_fp64 = ds.num_sms * tile_ctas_per_sm<false>();
+    const int g_fp64 = ds.num_sms * (tracers ? tile_ctas_per_sm<false, true>() : tile_ctas_per_sm<false>());
     if (mixed && tracers)
         batch_lsrk_noalloc_kernel<true, true><<<g_mixed, kThreads, tile_smem_bytes<true, true>(), s>>>(
             ds.scratch, kCoef, nsteps, dt);

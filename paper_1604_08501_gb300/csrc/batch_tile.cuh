@@ -9,6 +9,7 @@
 
 #include "element_sweep.cuh"
 #include "eos.cuh"
+#include "fixed_sweep.cuh"
 #include "numa_internal.h"
 
 namespace numa {
@@ -18,8 +19,13 @@ namespace {
 constexpr int kThreads = 512;
 
 // Shared memory of one CTA and CTAs per SM.  FP64: the fluxes (15 values per
-// thread); q and dq stay in registers and one CTA holds an SM (the FP64 pipe
-// binds).  Mixed: the fluxes, q and dq (10 values) and the point's geometry
+// thread), q and dq (10 values); the D sweeps run on the integer pipes
+// (fixed_sweep.cuh), so two CTAs of 64 registers share an SM and one's sweeps
+// run beside the other's FP64 phases (the FP64 pipe binds, about 72 operations
+// per point and stage).  Measured on 6 instances, 4.6 million points, ten steps
+// (50 stages): 75.5 ms with FP64 sweeps, q and dq in registers and one CTA per SM,
+// 36.5 ms so.  The tracer form keeps the base fields' q and dq in registers
+// (98 KB of fluxes: one CTA per SM).  Mixed: the fluxes, q and dq (10 values) and the point's geometry
 // (g and Jinv, 10 values) in shared memory, so that the kernel fits 64
 // registers and two CTAs share an SM, twice the warps to hide latency.
 // Flux words of one pass: 3 x NF blocks of EPP elements; the largest over the
@@ -42,16 +48,32 @@ __host__ __device__ constexpr int tile_flux_words() {
 }
 constexpr int kMixedFluxWords = tile_flux_words<float>();
 constexpr int kMixedSmemWords = kMixedFluxWords + (2 * 5 + 10) * kThreads;
+// FP64: the exponents of the lines' fixed-point sums (fixed_sweep.cuh) follow.
+template <int NF>
+__host__ __device__ constexpr int tile_lines() {   // lines of one pass: the largest over the orders
+    int m = 0;
+    for (int nq = 2; nq <= 8; ++nq) {
+        const int x = 3 * NF * (kThreads / (nq * nq * nq)) * nq * nq;
+        m = x > m ? x : m;
+    }
+    return m;
+}
+// State words per thread in shared memory in FP64: q and dq of every field, or
+// of the tracers alone in the tracer form.
+template <bool TR>
+__host__ __device__ constexpr int fp64_state_words() {
+    return TR ? 2 * (kMaxFields - kFields) : 2 * kFields;
+}
 template <bool MIXED, bool TR = false>
 constexpr size_t tile_smem_bytes() {
     constexpr int NF = TR ? kMaxFields : kFields;
     return MIXED ? sizeof(float) * (tile_flux_words<float, NF>() + (2 * NF + 10) * kThreads)
-                 : sizeof(double) * (tile_flux_words<double, NF>() +
-                                     (TR ? 2 * (kMaxFields - kFields) * kThreads : 0));
+                 : sizeof(double) * (tile_flux_words<double, NF>() + fp64_state_words<TR>() * kThreads) +
+                       sizeof(short) * tile_lines<NF>();
 }
-template <bool MIXED>
+template <bool MIXED, bool TR = false>
 constexpr int tile_ctas_per_sm() {
-    return MIXED ? 2 : 1;
+    return MIXED || !TR ? 2 : 1;
 }
 
 // Sweep tables per Nq (index Nq; 2..8 used).  They depend only on the order:
@@ -64,16 +86,19 @@ struct SweepTables {
 };
 __constant__ SweepTables<double> c_sweep64[9];
 __constant__ SweepTables<float> c_sweep32[9];
+__constant__ FixedTables<16, 4> c_fixed[9];
 
 // Fills this translation unit's tables on the current device (synchronous).
 inline cudaError_t upload_sweep_tables() {
     SweepTables<double> t64[9] = {};
     SweepTables<float> t32[9] = {};
+    FixedTables<16, 4> tf[9] = {};
     for (int N = 1; N <= 7; ++N) {
         double D[64];
         gll_diff_matrix(N, D);
         SweepTables<double> &a = t64[N + 1];
         sweep_tables(N, D, a.De, a.Do, a.Dc, a.Dcr);
+        fixed_tables(N, D, &tf[N + 1]);
         SweepTables<float> &b = t32[N + 1];
         for (int t = 0; t < 16; ++t) {
             b.De[t] = static_cast<float>(a.De[t]);
@@ -86,6 +111,7 @@ inline cudaError_t upload_sweep_tables() {
     }
     cudaError_t e = cudaMemcpyToSymbol(c_sweep64, t64, sizeof(t64));
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_sweep32, t32, sizeof(t32));
+    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_fixed, tf, sizeof(tf));
     return e;
 }
 
@@ -119,8 +145,12 @@ __device__ void run_tile(const BatchInstance &I, int64_t e0, int64_t count,
     constexpr int EW = block_words<NQ, T>();    // one element's (direction, field) block
     constexpr int BLK = EPP * EW;               // one (direction, field) block of sF
     constexpr int TASKS = 3 * NF * EPP * NL;    // lines per stage (TR: some blocks unused)
+    constexpr bool SMEM_STATE = MIXED || !TR;   // the base fields' q and dq
     const int nf = TR ? I.nf : kFields;
     T *sF = static_cast<T *>(smem);             // [(d*NF + b)*EPP + el][slot]
+    // FP64: the lines' exponents, [((d*NF + b)*EPP + el)*NL + line]
+    short *sE = reinterpret_cast<short *>(sF + tile_flux_words<T, NF>() +
+                                          fp64_state_words<TR>() * kThreads);
     const int l = threadIdx.x;
     const int el = l / N3, p = l % N3;
     const int i = p % NQ, j = (p / NQ) % NQ, k = p / NL;
@@ -145,8 +175,8 @@ __device__ void run_tile(const BatchInstance &I, int64_t e0, int64_t count,
         // shared memory in the mixed mode), and the mixed mode's per-point
         // constants, kept for all stages
         T qr[kFields], dqr[kFields];
-        T *sQ = sF + tile_flux_words<T, NF>() + l;   // [b * kThreads], mixed: every field
-        T *sD = sQ + NF * kThreads;                  // FP64 (TR): the tracers
+        T *sQ = sF + tile_flux_words<T, NF>() + l;   // [b * kThreads], every field
+        T *sD = sQ + NF * kThreads;                  // (FP64, TR: the tracers alone)
         T *sG = sD + NF * kThreads;                  // g (9), Jinv; mixed only
         // the tracers' q and dq (TR): shared memory in both precisions
         auto QT = [&](int t) -> T & {
@@ -158,10 +188,10 @@ __device__ void run_tile(const BatchInstance &I, int64_t e0, int64_t count,
             else return sF[tile_flux_words<T, NF>() + (NTR + t) * kThreads + l];
         };
         auto Q = [&](int b) -> T & {
-            if constexpr (MIXED) return sQ[b * kThreads]; else return qr[b];
+            if constexpr (SMEM_STATE) return sQ[b * kThreads]; else return qr[b];
         };
         auto DQ = [&](int b) -> T & {
-            if constexpr (MIXED) return sD[b * kThreads]; else return dqr[b];
+            if constexpr (SMEM_STATE) return sD[b * kThreads]; else return dqr[b];
         };
 #pragma unroll
         for (int b = 0; b < kFields; ++b) {
@@ -252,7 +282,8 @@ __device__ void run_tile(const BatchInstance &I, int64_t e0, int64_t count,
                         if constexpr (MIXED)
                             sweep_line<NQ>(sF + bd * BLK + e * EW, line, c_sweep32[NQ]);
                         else
-                            sweep_line<NQ>(sF + bd * BLK + e * EW, line, c_sweep64[NQ]);
+                            sE[t] = (short)sweep_line_fixed<NQ>(sF + bd * BLK + e * EW, line,
+                                                                c_sweep64[NQ], c_fixed[NQ]);
                     }
                 }
                 // FP64: J^-1 and rho_ref loaded before the barrier, so that
@@ -266,6 +297,18 @@ __device__ void run_tile(const BatchInstance &I, int64_t e0, int64_t count,
                 }
                 __syncthreads();
                 // ---- phase 3: rhs, stage update ------------------------
+                // the sum of field b's three sweeps at the thread's point
+                auto sum3 = [&](int b) -> T {
+                    const T r = sF[f[0] + b * BLK], s = sF[f[1] + b * BLK], t = sF[f[2] + b * BLK];
+                    if constexpr (MIXED) {
+                        return r + s + t;
+                    } else {
+                        constexpr int EB = EPP * NL;   // lines of one (direction, field)
+                        const short *E = sE + b * EB + el * NL;
+                        return fixed_sum3<NQ>(r, E[NQ * k + j], s, E[NF * EB + NQ * k + i], t,
+                                              E[2 * NF * EB + NQ * j + i], c_fixed[NQ].shift);
+                    }
+                };
                 if (active) {
                     const T a = sco[st], bcoef = sco[5 + st];
                     T jinv, drho;   // drho: rho - rho_ref of this stage's state, before the update
@@ -278,7 +321,7 @@ __device__ void run_tile(const BatchInstance &I, int64_t e0, int64_t count,
                     }
 #pragma unroll
                     for (int b = 0; b < kFields; ++b) {
-                        const T R = sF[f[0] + b * BLK] + sF[f[1] + b * BLK] + sF[f[2] + b * BLK];
+                        const T R = sum3(b);
                         T rhs = -jinv * R;
                         if (b == 3) rhs = fma(-drho, grav, rhs);
                         const T d = fma(a, DQ(b), dtt * rhs);
@@ -290,7 +333,7 @@ __device__ void run_tile(const BatchInstance &I, int64_t e0, int64_t count,
                         for (int t = 0; t < NTR; ++t) {
                             if (kFields + t >= nf) break;
                             const int b = kFields + t;
-                            const T R = sF[f[0] + b * BLK] + sF[f[1] + b * BLK] + sF[f[2] + b * BLK];
+                            const T R = sum3(b);
                             const T d = fma(a, DQT(t), dtt * (-jinv * R));
                             DQT(t) = d;
                             QT(t) = fma(bcoef, d, QT(t));
@@ -309,6 +352,22 @@ __device__ void run_tile(const BatchInstance &I, int64_t e0, int64_t count,
             }
         }
     }
+}
+
+// A function of its own per order (not inlined): each tile is then
+// register-allocated by itself (inlined together the FP64 tiles spill).
+template <int NQ, bool MIXED, bool TR>
+__device__ __noinline__ void run_tile_call(const BatchInstance &I, int64_t e0, int64_t count,
+                                           const tile_t<MIXED> *sco, int nsteps, double dt,
+                                           void *smem) {
+    run_tile<NQ, MIXED, TR>(I, e0, count, sco, nsteps, dt, smem);
+}
+template <int NQ, bool MIXED, bool TR>
+__device__ __forceinline__ void run_tile_either_way(const BatchInstance &I, int64_t e0,
+                                                    int64_t count, const tile_t<MIXED> *sco,
+                                                    int nsteps, double dt, void *smem) {
+    if constexpr (MIXED) run_tile<NQ, MIXED, TR>(I, e0, count, sco, nsteps, dt, smem);
+    else run_tile_call<NQ, MIXED, TR>(I, e0, count, sco, nsteps, dt, smem);
 }
 
 }  // namespace

@@ -23,6 +23,10 @@
 // S_i = sum_n D[i][n] F_n.
 #pragma once
 
+#include <cmath>
+
+#include <cuda_runtime.h>
+
 namespace numa {
 
 // Words between consecutive lines: for 4-byte values at Nq >= 8 the smallest
@@ -42,7 +46,7 @@ __host__ __device__ constexpr int block_words() {
 }
 
 template <int NQ, typename T>
-__device__ __forceinline__ int slot(int line, int n) {
+__host__ __device__ __forceinline__ int slot(int line, int n) {
     if constexpr (NQ >= 8 && sizeof(T) == 4)   // lines of an odd number of slots
         return line * line_stride<NQ, T>() + n;
     else if constexpr (NQ > 8)   // lines padded to 16 slots, XOR swizzle over 16
@@ -77,7 +81,7 @@ __device__ __forceinline__ int dir_slot(int d, int i, int j, int k) {
 // D[r][c] and Dcr[m] = D[c][m] for odd Nq.  The tables live in kernel
 // parameter space, so every thread reads the same constant-bank operand.
 template <int NQ, typename T, typename Tab>
-__device__ __forceinline__ void sweep_line(T *buf, int line, const Tab &tab) {
+__host__ __device__ __forceinline__ void sweep_line(T *buf, int line, const Tab &tab) {
     constexpr int HALF = NQ / 2;
     constexpr bool ODD = (NQ & 1) != 0;
     constexpr int C = NQ / 2;

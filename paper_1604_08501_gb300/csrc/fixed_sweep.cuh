@@ -1,0 +1,246 @@
+// The D sweep of one line of FP64 fluxes in 64-bit fixed point.
+//
+// GB300 issues 1.67 DFMA per clock and SM (measured) but about 30 multiply-adds of
+// 32 x 32 + 64 bits and 60 other integer operations, and an even-odd sweep in
+// FP64 (element_sweep.cuh) is 90 of the volume term's 157 FP64 operations per
+// point at Nq = 8.  Here the sums run on the integer pipes, beside the FP64
+// pipe, and are more accurate than in FP64:
+//
+//  * The thread of a line takes the largest exponent field e of its Nq fluxes
+//    and writes each as an integer X with F = X 2^(e - 1080), |X| < 2^58: the 53
+//    significant bits of the largest flux, and 5 bits below.
+//  * E_m = X_m + X_{N-m} and O_m = X_m - X_{N-m} are exact, below 2^59.
+//  * D is an integer too, D 2^s rounded to nearest, s such that the largest sum
+//    of |D[i][n]| over a row is at most 2^58.  Both are cut at bit 28 into
+//    32-bit words, E = Eh 2^28 + El (0 <= El < 2^28) and D = Dh 2^28 + Dl
+//    (|Dl| <= 2^27), and
+//      sum D E / 2^56 = sum Eh Dh + (sum (Eh Dl + El Dh)) / 2^28 + (sum El Dl) / 2^56.
+//    The first sum is exact (below 2^60), the second too (at most 9 terms below
+//    2^59 each) and its quotient is rounded down; the third, below 4.5, is
+//    dropped.  Three multiply-adds per product.
+//  * S_i = a_i + b_i and S_{N-i} = b_i - a_i, |S| <= 2^60, replace the line's
+//    fluxes; the value is S 2^(e - 1024 - s).  Phase 3 adds a point's three sums
+//    as integers at the largest of their exponents (|sum| <= 3 2^60) and rounds
+//    once to FP64.
+//
+// Measured: vol_rhs_fp64_kernel at N = 7, 32768 elements, 4.949 -> 1.881 ms; the
+// FP64 batch 2.07 times as fast.
+//
+// Error: at most 1 in each X and 2^-1 in each integer D entry, so at most
+// 2^-55 (largest |D| row sum) (largest flux of the line), as a bound; the
+// rounding errors of the FP64 sweep of such a line are 2^-53 of its partial
+// sums.  tests/test_fixed_sweep_host.py holds it to that bound and to at most
+// the FP64 sweep's error, over random, smooth and graded lines of every Nq.
+//
+// Nq = 2 keeps the FP64 sweep: its D is +-1/2, so that FP64 rounds only sums and
+// differences, and the fixed-point sum of three directions, cut at 2^-58 of the
+// largest line, was less exact (6.0e-18 against 8.7e-19 of the line's scale on
+// smooth lines, where the sums are far smaller than the fluxes).
+//
+// Lines whose largest exponent field is outside [kFixMinExp, kFixMaxExp]
+// (infinities, NaN, values that could overflow, lines of tiny values) take the
+// FP64 sweep: their exponent is kFixNone and the slots hold doubles.  A line
+// of zeros is a line of integer zeros.
+#pragma once
+
+#include <cstdint>
+#include <cstring>
+
+#include "element_sweep.cuh"
+#include "kernel_params.h"
+
+namespace numa {
+
+constexpr int kFixMinExp = 200, kFixMaxExp = 1900;
+constexpr int kFixNone = -1;      // exponent of a line left in FP64
+
+// Orders whose lines are swept in fixed point.
+template <int NQ>
+__host__ __device__ constexpr bool fixed_point() {
+    return NQ > 2;
+}
+
+__host__ __device__ __forceinline__ long long fix_bits(double x) {
+#ifdef __CUDA_ARCH__
+    return __double_as_longlong(x);
+#else
+    long long b;
+    std::memcpy(&b, &x, sizeof b);
+    return b;
+#endif
+}
+
+__host__ __device__ __forceinline__ double fix_double(long long b) {
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double(b);
+#else
+    double x;
+    std::memcpy(&x, &b, sizeof x);
+    return x;
+#endif
+}
+
+// x >> n for any n >= 0 (n >= 64: all sign bits).
+__host__ __device__ __forceinline__ long long fix_shr(long long x, int n) {
+#ifdef __CUDA_ARCH__
+    long long r;
+    asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));   // clamps n
+    return r;
+#else
+    return x >> (n > 63 ? 63 : n);
+#endif
+}
+
+__host__ __device__ __forceinline__ int fix_clz(unsigned long long x) {
+#ifdef __CUDA_ARCH__
+    return __clzll((long long)x);
+#else
+    return x ? __builtin_clzll(x) : 64;
+#endif
+}
+
+// X of the double with bits b, in a line of largest exponent field e: its
+// mantissa with the hidden bit at bit 57, shifted down by the difference of
+// the exponents (towards zero), with its sign.  Zeros and subnormals shift out.
+__host__ __device__ __forceinline__ long long fix_from_bits(long long b, int e) {
+    const uint32_t hi = (uint32_t)((unsigned long long)b >> 32);
+    const int d = e - (int)((hi >> 20) & 0x7FFu);
+    const long long m =
+        (long long)((((unsigned long long)((hi & 0xFFFFFu) | 0x100000u)) << 32 | (uint32_t)b)
+                    << (kFixBits - 53));
+    const long long a = fix_shr(m, d), s = b >> 63;
+    return (a ^ s) - s;
+}
+
+// The integer R, |R| < 2^63, times 2^(e - 1024 - s), rounded to nearest (ties
+// away from zero).  kFixMinExp and kFixMaxExp keep the result normal.
+__host__ __device__ __forceinline__ double fix_to_double(long long R, int e, int shift) {
+    const long long s = R >> 63;
+    const unsigned long long a = (unsigned long long)((R ^ s) - s);
+    const int lz = fix_clz(a);
+    const unsigned long long m = a << (lz & 63);   // leading bit at 63
+    // exponent field of 2^(63 - lz) 2^(e - 1024 - s), less the hidden bit's one
+    const int E = e - shift + 61 - lz;
+    const unsigned long long v = ((unsigned long long)(uint32_t)E << 52) + (m >> 11) + ((m >> 10) & 1ull);
+    return a == 0ull ? 0.0 : fix_double((long long)(v | ((unsigned long long)s & (1ull << 63))));
+}
+
+// The FP64 sweep, for the lines that cannot be fixed point.  Out of line: its
+// registers stay out of the kernels' budget.
+template <int NQ, typename Tab>
+__host__ __device__ __attribute__((noinline)) void sweep_line_fp64_call(double *buf, int line, const Tab &tab) {
+    sweep_line<NQ>(buf, line, tab);
+}
+
+// One product of a sum: acc_h += Eh Dh, acc_m += Eh Dl + El Dh.
+struct FixedSum {
+    long long h, m;
+};
+__host__ __device__ __forceinline__ void fix_mad(FixedSum &a, int Eh, int El, int Dh, int Dl) {
+    a.h += (long long)Eh * Dh;
+    a.m += (long long)Eh * Dl;
+    a.m += (long long)El * Dh;
+}
+__host__ __device__ __forceinline__ long long fix_value(FixedSum a) {
+    return a.h + (a.m >> kFixLow);
+}
+
+// X[0..NQ): the line's integers, replaced by its sums S.
+template <int NQ, typename FT>
+__host__ __device__ __forceinline__ void sweep_fixed(long long *X, const FT &ft) {
+    constexpr int HALF = NQ / 2;
+    constexpr bool ODD = (NQ & 1) != 0;
+    constexpr int C = NQ / 2;
+    constexpr long long MASK = (1ll << kFixLow) - 1;
+    int Eh[HALF], El[HALF], Oh[HALF], Ol[HALF];
+#pragma unroll
+    for (int m = 0; m < HALF; ++m) {
+        const long long E = X[m] + X[NQ - 1 - m], O = X[m] - X[NQ - 1 - m];
+        Eh[m] = (int)(E >> kFixLow);
+        El[m] = (int)(E & MASK);
+        Oh[m] = (int)(O >> kFixLow);
+        Ol[m] = (int)(O & MASK);
+    }
+    int Ch = 0, Cl = 0;
+    if constexpr (ODD) {
+        Ch = (int)(X[C] >> kFixLow);
+        Cl = (int)(X[C] & MASK);
+    }
+#pragma unroll
+    for (int r = 0; r < HALF; ++r) {
+        FixedSum a{0, 0}, b{0, 0};
+        if constexpr (ODD) fix_mad(a, Ch, Cl, ft.Dch[r], ft.Dcl[r]);
+#pragma unroll
+        for (int m = 0; m < HALF; ++m) {
+            fix_mad(a, Eh[m], El[m], ft.Deh[r * HALF + m], ft.Del[r * HALF + m]);
+            fix_mad(b, Oh[m], Ol[m], ft.Doh[r * HALF + m], ft.Dol[r * HALF + m]);
+        }
+        const long long A = fix_value(a), B = fix_value(b);
+        X[r] = B + A;
+        X[NQ - 1 - r] = B - A;
+    }
+    if constexpr (ODD) {
+        FixedSum c{0, 0};
+#pragma unroll
+        for (int m = 0; m < HALF; ++m) fix_mad(c, Oh[m], Ol[m], ft.Dcrh[m], ft.Dcrl[m]);
+        X[C] = fix_value(c);
+    }
+}
+
+// Sweep line `line` of buf in place: fluxes (doubles) in, integer sums out,
+// and the line's exponent returned (kFixNone: the sums are doubles).
+template <int NQ, typename Tab, typename FT>
+__host__ __device__ __forceinline__ int sweep_line_fixed(double *buf, int line, const Tab &tab, const FT &ft) {
+    if constexpr (!fixed_point<NQ>()) {
+        sweep_line<NQ>(buf, line, tab);
+        return kFixNone;
+    }
+    long long X[NQ];
+    uint32_t top = 0, any = 0;
+#pragma unroll
+    for (int n = 0; n < NQ; ++n) {
+        X[n] = fix_bits(buf[slot<NQ, double>(line, n)]);
+        const uint32_t h = (uint32_t)((unsigned long long)X[n] >> 32) & 0x7FFFFFFFu;
+        top = h > top ? h : top;
+        any |= (uint32_t)X[n];
+    }
+    int e = (int)(top >> 20);
+    if (e < kFixMinExp || e > kFixMaxExp) {
+        if ((top | any) != 0u) {
+            sweep_line_fp64_call<NQ>(buf, line, tab);
+            return kFixNone;
+        }
+        e = kFixMinExp;   // zeros of either sign: X = 0
+    }
+#pragma unroll
+    for (int n = 0; n < NQ; ++n) X[n] = fix_from_bits(X[n], e);
+    sweep_fixed<NQ>(X, ft);
+#pragma unroll
+    for (int n = 0; n < NQ; ++n) buf[slot<NQ, double>(line, n)] = fix_double(X[n]);
+    return e;
+}
+
+// The sum of a point's three directions where a line is in FP64 (rare).
+static __host__ __device__ __attribute__((noinline)) double fixed_sum3_slow(double r, int er, double s, int es, double t,
+                                                      int et, int shift) {
+    const double R = er < 0 ? r : fix_to_double(fix_bits(r), er, shift);
+    const double S = es < 0 ? s : fix_to_double(fix_bits(s), es, shift);
+    const double T = et < 0 ? t : fix_to_double(fix_bits(t), et, shift);
+    return R + S + T;
+}
+
+// The sum of a point's three directions, from the slots' bits (r, s, t) and
+// the lines' exponents.
+template <int NQ>
+__host__ __device__ __forceinline__ double fixed_sum3(double r, int er, double s, int es, double t,
+                                                      int et, int shift) {
+    if constexpr (!fixed_point<NQ>()) return r + s + t;
+    if ((er | es | et) < 0) return fixed_sum3_slow(r, er, s, es, t, et, shift);
+    const int m = er > es ? er : es, e = m > et ? m : et;
+    const long long R = fix_shr(fix_bits(r), e - er) +
+                        fix_shr(fix_bits(s), e - es) +
+                        fix_shr(fix_bits(t), e - et);
+    return fix_to_double(R, e, shift);
+}
+
+}  // namespace numa

@@ -91,4 +91,35 @@ void sweep_tables(int N, const double *D, double De[16], double Do[16], double D
     }
 }
 
+int fixed_tables(int N, const double *D, int *Deh, int *Del, int *Doh, int *Dol, int *Dch, int *Dcl,
+                 int *Dcrh, int *Dcrl) {
+    const int Nq = N + 1, half = Nq / 2, ctr = Nq / 2;
+    long double rows = 0.0L;
+    for (int i = 0; i < Nq; ++i) {
+        long double sum = 0.0L;
+        for (int n = 0; n < Nq; ++n) sum += std::fabs((long double)D[i * Nq + n]);
+        rows = sum > rows ? sum : rows;
+    }
+    int ex = 0;
+    std::frexp(rows, &ex);   // rows < 2^ex
+    const int shift = kFixBits - ex;
+    auto put = [shift](long double x, int *h, int *l) {
+        const long long v = std::llround(std::ldexp(x, shift));
+        *h = (int)((v + (1ll << (kFixLow - 1))) >> kFixLow);
+        *l = (int)(v - ((long long)*h << kFixLow));
+    };
+    for (int r = 0; r < half; ++r) {
+        for (int m = 0; m < half; ++m) {
+            const long double a = D[r * Nq + m], b = D[r * Nq + (Nq - 1 - m)];
+            put((a + b) / 2, &Deh[r * half + m], &Del[r * half + m]);
+            put((a - b) / 2, &Doh[r * half + m], &Dol[r * half + m]);
+        }
+        if (Nq & 1) {
+            put(D[r * Nq + ctr], &Dch[r], &Dcl[r]);
+            put(D[ctr * Nq + r], &Dcrh[r], &Dcrl[r]);
+        }
+    }
+    return shift;
+}
+
 }  // namespace numa

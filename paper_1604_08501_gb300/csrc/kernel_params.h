@@ -34,10 +34,22 @@ struct EosConstants {
     double p0, R, gamma, grav;
 };
 
+// Even-odd tables of D 2^shift as (high, low) integer words for the fixed-point
+// sweep of the FP64 kernels (fixed_sweep.cuh); T: entries of De and Do, H: of
+// the centre column and row (odd Nq).
+constexpr int kFixBits = 58;   // line values are integers below 2^58, row sums of |D| 2^shift at most that
+constexpr int kFixLow = 28;    // bits of the low words
+template <int T, int H>
+struct FixedTables {
+    int Deh[T], Del[T], Doh[T], Dol[T], Dch[H], Dcl[H], Dcrh[H], Dcrl[H];
+    int shift;
+};
+
 // Parameters of the native kernel: EOS constants, c[k] = binom(gamma, k+1)
 // (k = 0..14, the coefficients of the p' series), and the even-odd pieces of D
 // for r, m < Nq/2: De = (D[r][m] + D[r][N-m])/2, Do = (D[r][m] - D[r][N-m])/2,
-// Dc[r] = D[r][c] and Dcr[m] = D[c][m] (centre column and row, odd Nq).
+// Dc[r] = D[r][c] and Dcr[m] = D[c][m] (centre column and row, odd Nq).  (The
+// integer tables go beside it: a batch keeps a NativeParams per instance.)
 // Uniform across threads, so the kernel reads them as constant-bank operands.
 struct NativeParams {
     EosConstants eos;
@@ -51,6 +63,7 @@ struct HighParams {
     EosConstants eos;
     double c[15];
     double De[64], Do[64], Dc[8], Dcr[8];
+    FixedTables<64, 8> fix;
 };
 
 // The same for the mixed-precision mode at N = 8..15: FP32 tables and the FP32

@@ -28,8 +28,8 @@ cudaError_t launch_vol_rhs_mixed_high(int N, int nf, ElemRange r, const MixedGeo
                                       const HighParams32 &P, const float *q, float *rhs,
                                       int num_sms, cudaStream_t s);
 cudaError_t launch_vol_rhs_fp64(int N, int nf, ElemRange r, const DeviceGeometry &geo,
-                                const NativeParams &P, const double *q, double *rhs,
-                                cudaStream_t s);
+                                const NativeParams &P, const FixedTables<16, 4> &fix,
+                                const double *q, double *rhs, cudaStream_t s);
 
 // Launchers of the double-float path (vol_df64.cu).  abs_max: max |src| into
 // *amax_bits (the bit pattern of a nonnegative double).  to_df: split src
@@ -68,6 +68,16 @@ int gll_diff_matrix(int N, double *D);
 // ((Nq/2)^2, row-major), Dc, Dcr (odd Nq).  Unused entries are zero.
 void sweep_tables(int N, const double *D, double De[16], double Do[16], double Dc[4],
                   double Dcr[4]);
+
+// The same tables as integers D 2^shift, cut into (high, low) words at bit
+// kFixLow (fixed_sweep.cuh): the arrays of a FixedTables; the shift is returned.
+int fixed_tables(int N, const double *D, int *Deh, int *Del, int *Doh, int *Dol, int *Dch, int *Dcl,
+                 int *Dcrh, int *Dcrl);
+template <int T, int H>
+void fixed_tables(int N, const double *D, FixedTables<T, H> *f) {
+    *f = FixedTables<T, H>{};
+    f->shift = fixed_tables(N, D, f->Deh, f->Del, f->Doh, f->Dol, f->Dch, f->Dcl, f->Dcrh, f->Dcrl);
+}
 
 // Native: vol_rhs_fp64_kernel (N <= 7); NativeHigh: vol_rhs_high_kernel<Nq, double>
 // (N = 8..15); DoubleFloat (vol_rhs_df64_kernel<Nq>, N <= 7); Mixed (N <= 7) and MixedHigh:
@@ -153,6 +163,7 @@ struct numa_vol {
     numa::DfGeometry dgeo{};        // double-float path
     numa::DfParams dparams{};
     numa::NativeParams nparams{};
+    numa::FixedTables<16, 4> nfix{};   // the integer tables beside nparams
     numa::HighParams hparams{};      // NUMA_FP64, N >= 8
     numa::HighParams32 hmparams{};   // NUMA_MIXED, N >= 8
     numa::MixedGeometry mgeo{};     // mixed-precision path

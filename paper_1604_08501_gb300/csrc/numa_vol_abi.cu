@@ -142,6 +142,7 @@ void build_params(numa_vol *h, const double *D) {
         h->hparams.eos = h->eos;
         for (int k = 0; k < 15; ++k) h->hparams.c[k] = h->nparams.c[k];
         numa::sweep_tables(h->N, D, h->hparams.De, h->hparams.Do, h->hparams.Dc, h->hparams.Dcr);
+        numa::fixed_tables(h->N, D, &h->hparams.fix);
         numa::HighParams32 &m = h->hmparams;
         for (int t = 0; t < 64; ++t) {
             m.De[t] = static_cast<float>(h->hparams.De[t]);
@@ -159,6 +160,7 @@ void build_params(numa_vol *h, const double *D) {
         return;
     }
     numa::sweep_tables(h->N, D, h->nparams.De, h->nparams.Do, h->nparams.Dc, h->nparams.Dcr);
+    numa::fixed_tables(h->N, D, &h->nfix);
     {
         numa::MixedParams &m = h->mparams;
         for (int t = 0; t < 16; ++t) {
@@ -450,7 +452,7 @@ cudaError_t launch(numa_vol *h, const void *q, void *rhs, int64_t e0, int64_t co
                                               static_cast<const double *>(q),
                                               static_cast<double *>(rhs), s);
     return numa::launch_vol_rhs_fp64(h->N, h->nf, r, h->geo, h->nparams,
-                                     static_cast<const double *>(q), static_cast<double *>(rhs), s);
+                                     h->nfix, static_cast<const double *>(q), static_cast<double *>(rhs), s);
 }
 
 }  // namespace

@@ -5,10 +5,12 @@
 // equation of state, the contravariant fluxes of the five fields in the three
 // reference directions, the three D sweeps, the Jinv scaling and the gravity
 // source (Sec. 2, Eq. (2); sign and flux form of the paper's r/s subroutines,
-// Sec. 3).  Every floating-point operation is an FP64 operation.
+// Sec. 3).  State, geometry, pressure, fluxes and rhs are FP64; the D sweeps
+// run in 64-bit fixed point (fixed_sweep.cuh), whose error is below the FP64
+// sweeps'.
 //
-// On GB300 the FP64 pipe (about 0.53 T DFMA/s) binds this kernel, so the
-// design minimises FP64 instructions per point:
+// On GB300 the FP64 pipe (1.67 DFMA per clock and SM, 0.53 T/s) binds this
+// kernel, so the design minimises FP64 instructions per point:
 //  * p' = p(Theta) - p(Theta_ref) is evaluated as p_ref ((1+x)^gamma - 1) by
 //    its binomial series in x = (Theta - Theta_ref)/Theta_ref (12 FP64
 //    operations for |x| <= 1/64, and no cancellation); eos.cuh has the wider
@@ -17,10 +19,14 @@
 //  * The fluxes are computed once per point into shared memory (the paper's
 //    flux precompute, Sec. 3, opt. level 5).
 //  * Each line of each (direction, field) is swept by one thread with the
-//    even-odd split of the GLL D (D[N-i][N-n] = -D[i][n]): E_m = F_m + F_{N-m},
-//    O_m = F_m - F_{N-m}, and S_i = a_i + b_i, S_{N-i} = b_i - a_i with
-//    a_i = sum_m De[i][m] E_m (+ D[i][c] F_c for odd Nq), b_i = sum_m Do[i][m] O_m.
-//    That is half the multiplies of the direct sweep.
+//    even-odd split of the GLL D (D[N-i][N-n] = -D[i][n]), half the multiplies
+//    of the direct sweep, on the integer pipes: no FP64 operation.  The sweeps
+//    and the sums over the directions were 100 of 157 FP64 operations per point
+//    at Nq = 8.  One thread's integers take 64 registers, as two CTAs of 512
+//    threads allow, and the integer work of one CTA runs beside the FP64 work
+//    of the other.  Measured at N = 7, 32768 elements: 4.949 ms with FP64
+//    sweeps, 1.881 ms (59 FP64 operations' time per point) in fixed point;
+//    N = 4, 512 elements, a call among others: 22.5 and 14.3 us.
 //  * Jinv is applied once to the sum of the three sweeps (opt. level 8).
 //
 // One CTA of Nq^3 threads per element, in three phases: fluxes by point,
@@ -29,6 +35,7 @@
 
 #include "element_sweep.cuh"
 #include "eos.cuh"
+#include "fixed_sweep.cuh"
 #include "numa_internal.h"
 
 namespace numa {
@@ -47,12 +54,14 @@ constexpr int min_ctas() {
 // Theta with flux Q u_d and no source.  Without tracers nf is 5.
 template <int NQ, bool TRACERS>
 __global__ void __launch_bounds__(NQ * NQ * NQ, min_ctas<NQ>())
-vol_rhs_fp64_kernel(DeviceGeometry geo, NativeParams P, const double *__restrict__ q,
-                    double *__restrict__ rhs, int64_t M, int64_t e0, int nf_run) {
+vol_rhs_fp64_kernel(DeviceGeometry geo, const __grid_constant__ NativeParams P,
+                    FixedTables<16, 4> fix, const double *__restrict__ q, double *__restrict__ rhs, int64_t M, int64_t e0,
+                    int nf_run) {
     constexpr int N3 = NQ * NQ * NQ;
     constexpr int NL = NQ * NQ;               // lines per (direction, field)
     const int nf = TRACERS ? nf_run : kFields;
     extern __shared__ double sF[];            // [direction*nf + field][slot]
+    short *sE = reinterpret_cast<short *>(sF + 3 * nf * N3);   // [direction*nf + field][line]
 
     const int l = threadIdx.x;
     const int i = l % NQ, j = (l / NQ) % NQ, k = l / (NQ * NQ);
@@ -93,7 +102,7 @@ vol_rhs_fp64_kernel(DeviceGeometry geo, NativeParams P, const double *__restrict
 
     // ---- phase 2: even-odd sweeps, one line per task, in place --------
     for (int item = l; item < 3 * nf * NL; item += N3)
-        sweep_line<NQ>(sF + (item / NL) * N3, item % NL, P);
+        sE[item] = (short)sweep_line_fixed<NQ>(sF + (item / NL) * N3, item % NL, P, fix);
     __syncthreads();
 
     // ---- phase 3: combine, scale, gravity, store ----------------------
@@ -102,9 +111,12 @@ vol_rhs_fp64_kernel(DeviceGeometry geo, NativeParams P, const double *__restrict
 #pragma unroll
     for (int b = 0; b < (TRACERS ? kMaxFields : kFields); ++b) {
         if (TRACERS && b >= nf) break;
-        const double R = sF[(0 * nf + b) * N3 + dir_slot<NQ, double>(0, i, j, k)] +
-                         sF[(1 * nf + b) * N3 + dir_slot<NQ, double>(1, i, j, k)] +
-                         sF[(2 * nf + b) * N3 + dir_slot<NQ, double>(2, i, j, k)];
+        const double R = fixed_sum3<NQ>(sF[(0 * nf + b) * N3 + dir_slot<NQ, double>(0, i, j, k)],
+                                    sE[(0 * nf + b) * NL + NQ * k + j],
+                                    sF[(1 * nf + b) * N3 + dir_slot<NQ, double>(1, i, j, k)],
+                                    sE[(1 * nf + b) * NL + NQ * k + i],
+                                    sF[(2 * nf + b) * N3 + dir_slot<NQ, double>(2, i, j, k)],
+                                    sE[(2 * nf + b) * NL + NQ * j + i], fix.shift);
         double v = -Jinv * R;
         if (b == 3) v = fma(-drho, P.eos.grav, v);
         rhs[b * M + node] = v;
@@ -113,24 +125,24 @@ vol_rhs_fp64_kernel(DeviceGeometry geo, NativeParams P, const double *__restrict
 
 template <int NQ, bool TRACERS>
 cudaError_t launch_kernel(ElemRange r, int nf, const DeviceGeometry &geo, const NativeParams &P,
-                          const double *q, double *rhs, cudaStream_t s) {
+                          const FixedTables<16, 4> &fix, const double *q, double *rhs, cudaStream_t s) {
     constexpr int N3 = NQ * NQ * NQ;
-    const size_t smem = sizeof(double) * nf * 3 * N3;
+    const size_t smem = (sizeof(double) * N3 + sizeof(short) * NQ * NQ) * nf * 3;
     // The opt-in above 48 KB is per device; setting it on every launch keeps
     // multi-device processes correct and costs about a microsecond.
     cudaError_t e = cudaFuncSetAttribute(vol_rhs_fp64_kernel<NQ, TRACERS>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    vol_rhs_fp64_kernel<NQ, TRACERS><<<(unsigned)r.count, N3, smem, s>>>(geo, P, q, rhs, r.M, r.e0,
-                                                                         nf);
+    vol_rhs_fp64_kernel<NQ, TRACERS><<<(unsigned)r.count, N3, smem, s>>>(geo, P, fix, q, rhs, r.M,
+                                                                         r.e0, nf);
     return cudaGetLastError();
 }
 
 template <int NQ>
 cudaError_t launch_nq(ElemRange r, int nf, const DeviceGeometry &geo, const NativeParams &P,
-                      const double *q, double *rhs, cudaStream_t s) {
-    if (nf == kFields) return launch_kernel<NQ, false>(r, nf, geo, P, q, rhs, s);
-    return launch_kernel<NQ, true>(r, nf, geo, P, q, rhs, s);
+                      const FixedTables<16, 4> &fix, const double *q, double *rhs, cudaStream_t s) {
+    if (nf == kFields) return launch_kernel<NQ, false>(r, nf, geo, P, fix, q, rhs, s);
+    return launch_kernel<NQ, true>(r, nf, geo, P, fix, q, rhs, s);
 }
 
 // w = 1/Theta_ref and A = p(Theta_ref)/Theta_ref, in place of a copy of Theta_ref.
@@ -154,18 +166,18 @@ cudaError_t launch_reference_eos(const double *theta_ref, double *w, double *A, 
 }
 
 cudaError_t launch_vol_rhs_fp64(int N, int nf, ElemRange r, const DeviceGeometry &geo,
-                                const NativeParams &P, const double *q, double *rhs,
-                                cudaStream_t s) {
+                                const NativeParams &P, const FixedTables<16, 4> &fix,
+                                const double *q, double *rhs, cudaStream_t s) {
     if (r.count <= 0) return cudaSuccess;
     if (nf < kFields || nf > kMaxFields) return cudaErrorInvalidValue;
     switch (N) {
-        case 1: return launch_nq<2>(r, nf, geo, P, q, rhs, s);
-        case 2: return launch_nq<3>(r, nf, geo, P, q, rhs, s);
-        case 3: return launch_nq<4>(r, nf, geo, P, q, rhs, s);
-        case 4: return launch_nq<5>(r, nf, geo, P, q, rhs, s);
-        case 5: return launch_nq<6>(r, nf, geo, P, q, rhs, s);
-        case 6: return launch_nq<7>(r, nf, geo, P, q, rhs, s);
-        case 7: return launch_nq<8>(r, nf, geo, P, q, rhs, s);
+        case 1: return launch_nq<2>(r, nf, geo, P, fix, q, rhs, s);
+        case 2: return launch_nq<3>(r, nf, geo, P, fix, q, rhs, s);
+        case 3: return launch_nq<4>(r, nf, geo, P, fix, q, rhs, s);
+        case 4: return launch_nq<5>(r, nf, geo, P, fix, q, rhs, s);
+        case 5: return launch_nq<6>(r, nf, geo, P, fix, q, rhs, s);
+        case 6: return launch_nq<7>(r, nf, geo, P, fix, q, rhs, s);
+        case 7: return launch_nq<8>(r, nf, geo, P, fix, q, rhs, s);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -54,7 +54,7 @@ def diff_matrix(N: int) -> np.ndarray:
 class VolumeTerm:
     """One mesh on the current CUDA device (numa_vol_create ... numa_vol_destroy).
 
-    precision: "fp64" (every operation on the FP64 pipe), "df64" (double-float
+    precision: "fp64" (FP64 arithmetic, the D sums no less exact), "df64" (double-float
     arithmetic on the FP32 pipes, N = 7) or "mixed" (FP32 perturbation state,
     see workload.perturbation_state)."""
 
