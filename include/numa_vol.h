@@ -100,7 +100,7 @@ typedef struct {
 
 typedef enum {
     NUMA_FP64 = 0,   /* FP64 state and rhs, FP64 arithmetic; the D sums in 64-bit
-                        fixed point (N >= 2, N <= 7), no less exact              */
+                        fixed point (N >= 2), no less exact                      */
     NUMA_MIXED = 1,  /* FP32 perturbation state (rho', U1, U2, U3, Theta'), FP32 rhs,
                         FP32 geometry and arithmetic                                    */
     NUMA_DF64 = 2    /* FP64 state and rhs, double-float arithmetic (hi + lo FP32 pairs,

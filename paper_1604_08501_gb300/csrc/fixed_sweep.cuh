@@ -145,9 +145,9 @@ __host__ __device__ __forceinline__ long long fix_value(FixedSum a) {
     return a.h + (a.m >> kFixLow);
 }
 
-// X[0..NQ): the line's integers, replaced by its sums S.
-template <int NQ, typename FT>
-__host__ __device__ __forceinline__ void sweep_fixed(long long *X, const FT &ft) {
+// The sums S of the line's integers X[0..NQ), each given to put(n, S) as it is formed.
+template <int NQ, typename FT, typename Put>
+__host__ __device__ __forceinline__ void sweep_fixed(const long long *X, const FT &ft, Put put) {
     constexpr int HALF = NQ / 2;
     constexpr bool ODD = (NQ & 1) != 0;
     constexpr int C = NQ / 2;
@@ -176,14 +176,14 @@ __host__ __device__ __forceinline__ void sweep_fixed(long long *X, const FT &ft)
             fix_mad(b, Oh[m], Ol[m], ft.Doh[r * HALF + m], ft.Dol[r * HALF + m]);
         }
         const long long A = fix_value(a), B = fix_value(b);
-        X[r] = B + A;
-        X[NQ - 1 - r] = B - A;
+        put(r, B + A);
+        put(NQ - 1 - r, B - A);
     }
     if constexpr (ODD) {
         FixedSum c{0, 0};
 #pragma unroll
         for (int m = 0; m < HALF; ++m) fix_mad(c, Oh[m], Ol[m], ft.Dcrh[m], ft.Dcrl[m]);
-        X[C] = fix_value(c);
+        put(C, fix_value(c));
     }
 }
 
@@ -214,9 +214,7 @@ __host__ __device__ __forceinline__ int sweep_line_fixed(double *buf, int line, 
     }
 #pragma unroll
     for (int n = 0; n < NQ; ++n) X[n] = fix_from_bits(X[n], e);
-    sweep_fixed<NQ>(X, ft);
-#pragma unroll
-    for (int n = 0; n < NQ; ++n) buf[slot<NQ, double>(line, n)] = fix_double(X[n]);
+    sweep_fixed<NQ>(X, ft, [&](int n, long long S) { buf[slot<NQ, double>(line, n)] = fix_double(S); });
     return e;
 }
 

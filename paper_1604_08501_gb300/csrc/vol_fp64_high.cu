@@ -24,8 +24,12 @@
 //    groups are large (five fields: four per group at Nq = 12, 13 and 16, one
 //    pass at the other orders; a separate form for tracers); after its first
 //    pass each CTA prefetches the element of the next wave to L2.
-// Shared memory at Nq = 16: 224 KB in FP64 (every operation FP64; bound by the
-// FP64 pipe like the low orders), 204 KB in the mixed mode (FP32 perturbation
+// The FP64 D sweeps run in 64-bit fixed point on the integer pipes
+// (fixed_sweep.cuh), as at the low orders: measured on 3.5 million points, five
+// fields, N = 11 1.405 -> 0.685 ms, N = 15 1.569 -> 0.839 ms, with three tracers
+// 2.100 -> 0.951 and 2.365 -> 1.200 ms; what is left is bound by the latency of
+// the passes' loads and barriers (a field at a time), no longer by the FP64 pipe.
+// Shared memory at Nq = 16: 226 KB in FP64, 204 KB in the mixed mode (FP32 perturbation
 // state and arithmetic as vol_mixed.cu).
 #include <cuda_runtime.h>
 
@@ -34,6 +38,7 @@
 #include "bulk_copy.cuh"
 #include "element_sweep.cuh"
 #include "eos.cuh"
+#include "fixed_sweep.cuh"
 #include "numa_internal.h"
 #include "tcgen05.cuh"
 
@@ -140,7 +145,8 @@ __host__ __device__ constexpr int high_group() {
 template <int NQ, typename T, int NF>
 __host__ __device__ constexpr size_t high_smem_bytes() {
     return sizeof(T) * ((sizeof(T) == 8 ? 4 * NQ * NQ * NQ : 0) +
-                        high_group<NQ, T, NF>() * 3 * NQ * NQ * line_stride<NQ, T>());
+                        high_group<NQ, T, NF>() * 3 * NQ * NQ * line_stride<NQ, T>()) +
+           (sizeof(T) == 8 ? sizeof(short) * high_group<NQ, T, NF>() * 3 * NQ * NQ : 0);
 }
 
 // CTAs per SM the register budget is sized for: two where two CTAs' shared
@@ -176,7 +182,8 @@ template <> struct HighTypes<float> { using Geo = MixedGeometry; using Params = 
 
 template <int NQ, typename T, int NF>
 __global__ void __launch_bounds__((high_threads<NQ, T>()), (high_min_ctas<NQ, T, NF>()))
-vol_rhs_high_kernel(typename HighTypes<T>::Geo geo, typename HighTypes<T>::Params P,
+vol_rhs_high_kernel(typename HighTypes<T>::Geo geo,
+                    const __grid_constant__ typename HighTypes<T>::Params P,
                     const T *__restrict__ q, T *__restrict__ rhs, int64_t M, int64_t e0, int nf,
                     int64_t e_end, int64_t ahead) {
     constexpr bool MIXED = sizeof(T) == 4;
@@ -199,6 +206,7 @@ vol_rhs_high_kernel(typename HighTypes<T>::Geo geo, typename HighTypes<T>::Param
     T *sU = reinterpret_cast<T *>(smem_raw);   // FP64: u_d of every point: [d][k][j][i]
     T *sP = sU + 3 * N3;                       // FP64: p' of every point: [k][j][i]
     T *sF = MIXED ? sU : sU + 4 * N3;          // fluxes of a group: [field][d][line][slot]
+    short *sE = reinterpret_cast<short *>(sF + G * 3 * FB);   // FP64: the lines' exponents, [field][d][line]
 
     const int t = threadIdx.x;
     const int c = t % NL, slab = t / NL;   // slab == TPC: a padding thread
@@ -404,7 +412,13 @@ vol_rhs_high_kernel(typename HighTypes<T>::Geo geo, typename HighTypes<T>::Param
         if constexpr (TPC == 3) {
             if (slab < 3) {
 #pragma unroll 1
-                for (int gl = 0; gl < gn; ++gl) sweep_line<NQ>(sF + (gl * 3 + slab) * FB, c, P);
+                for (int gl = 0; gl < gn; ++gl) {
+                    if constexpr (MIXED)
+                        sweep_line<NQ>(sF + (gl * 3 + slab) * FB, c, P);
+                    else
+                        sE[(gl * 3 + slab) * NL + c] =
+                            (short)sweep_line_fixed<NQ>(sF + (gl * 3 + slab) * FB, c, P, P.fix);
+                }
             }
         } else {
 #pragma unroll 1
@@ -444,7 +458,15 @@ vol_rhs_high_kernel(typename HighTypes<T>::Geo geo, typename HighTypes<T>::Param
                     if (gl >= gn) break;
                     const int b = b0 + gl;
                     const T *F = sF + gl * 3 * FB;
-                    T v = -jinv * (F[s0] + F[FB + s1] + F[2 * FB + s2]);
+                    T R;
+                    if constexpr (MIXED) {
+                        R = F[s0] + F[FB + s1] + F[2 * FB + s2];
+                    } else {
+                        const short *E = sE + gl * 3 * NL;
+                        R = fixed_sum3<NQ>(F[s0], E[NQ * k + j], F[FB + s1], E[NL + NQ * k + i],
+                                           F[2 * FB + s2], E[2 * NL + NQ * j + i], P.fix.shift);
+                    }
+                    T v = -jinv * R;
                     if (b == 3) {
                         if constexpr (MIXED)
                             v = fma(-rv[kk], P.grav, v);
