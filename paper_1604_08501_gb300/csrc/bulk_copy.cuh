@@ -33,6 +33,14 @@ __device__ __forceinline__ void prefetch_l2(const void *src_gmem, uint32_t bytes
                  : "memory");
 }
 
+// The same for any range inside an array whose start is 16-byte aligned: the
+// 16-byte units from the one that holds its first byte to the last whole one.
+__device__ __forceinline__ void prefetch_l2_units(const void *src_gmem, uint32_t bytes) {
+    const uint64_t a = reinterpret_cast<uint64_t>(src_gmem), first = a & ~15ull;
+    const uint32_t n = (uint32_t)((a + bytes) - first) & ~15u;
+    if (n) prefetch_l2(reinterpret_cast<const void *>(first), n);
+}
+
 // One poll of phase `parity` of `bar`; the thread may be suspended for up to
 // about hint_ns while the phase is incomplete.
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity, uint32_t hint_ns = 1000) {

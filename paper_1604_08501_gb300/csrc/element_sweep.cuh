@@ -57,6 +57,35 @@ __host__ __device__ __forceinline__ int slot(int line, int n) {
         return line * NQ + n;
 }
 
+// Threads of an element in the single-evaluation kernels of N <= 7: whole warps,
+// so that no warp holds points of two elements (the form of the equation of
+// state is chosen per warp, and an element's result depends on it alone), but
+// 8 at Nq = 2, where the four elements of a warp choose apart.
+template <int NQ>
+__host__ __device__ constexpr int element_threads() {
+    return NQ == 2 ? 8 : (NQ * NQ * NQ + 31) / 32 * 32;
+}
+// Elements per CTA: CTAs of 256 threads at Nq = 2, 3 and 4, one element from
+// Nq = 5.  An SM holds 32 CTAs, a quarter of its threads where a CTA is one
+// Nq = 2 element: 96^3 of them, one and 32 a CTA, take 449 and 99 us in
+// NUMA_MIXED, 6.10 and 1.50 ms in NUMA_FP64; 64^3 at Nq = 3 141 and 121 us (one
+// and 8 a CTA, the L2 prefetch with them); Nq = 4 is the same either way.  Two and
+// four elements a CTA at Nq = 5 and 6 were slower (N = 4, 54.7 to 65 us against
+// 53.4; N = 5 61.6 against 54.2): the CTA's barriers wait for more warps.
+template <int NQ>
+__host__ __device__ constexpr int cta_elements() {
+    return NQ == 2 ? 32 : NQ == 3 ? 8 : NQ == 4 ? 4 : 1;
+}
+template <int NQ>
+__host__ __device__ constexpr int cta_threads() {   // one element: a thread per point, no padding
+    return cta_elements<NQ>() == 1 ? NQ * NQ * NQ : cta_elements<NQ>() * element_threads<NQ>();
+}
+// Lanes of a warp that choose the form of the equation of state together.
+template <int NQ>
+__host__ __device__ constexpr int vote_lanes() {
+    return NQ == 2 ? 8 : 32;
+}
+
 // Slot of point (i, j, k) in direction d's block.  For 4-byte values at Nq = 8
 // (lines of 9 slots) the r and s lines are numbered so that a warp of points
 // (i = 0..7, four consecutive j, one k) touches 32 distinct banks in every
@@ -77,6 +106,56 @@ __device__ __forceinline__ int dir_slot(int d, int i, int j, int k) {
     }
 }
 
+// Values of a line one shared-memory access moves: 16 bytes where the lines are
+// whole 16-byte units (4-byte values at Nq = 4, 8-byte ones at Nq = 2, 4 and 6),
+// 8 bytes for 4-byte values at Nq = 2 and 6, else one value.  A warp's lines are
+// then read and written without bank conflicts but for 8-byte values at Nq = 4
+// (2-way; 4-way value by value).
+template <int NQ, typename T>
+__host__ __device__ constexpr int line_vector() {
+    if (NQ >= 8 || (NQ & 1)) return 1;
+    return sizeof(T) == 8 ? 2 : (NQ == 4 ? 4 : 2);
+}
+
+// F[0..NQ) = line `line` of buf.  buf is 16-byte aligned.
+template <int NQ, typename T>
+__host__ __device__ __forceinline__ void load_line(const T *buf, int line, T *F) {
+    constexpr int V = line_vector<NQ, T>();
+    if constexpr (V == 1) {
+#pragma unroll
+        for (int n = 0; n < NQ; ++n) F[n] = buf[slot<NQ, T>(line, n)];
+    } else {
+        struct alignas(V * sizeof(T)) Vec { T x[V]; };
+        const Vec *p = reinterpret_cast<const Vec *>(buf + line * NQ);
+#pragma unroll
+        for (int n = 0; n < NQ / V; ++n) {
+            const Vec v = p[n];
+#pragma unroll
+            for (int m = 0; m < V; ++m) F[n * V + m] = v.x[m];
+        }
+    }
+}
+
+// Line `line` of buf = S[0..NQ).
+template <int NQ, typename T>
+__host__ __device__ __forceinline__ void store_line(T *buf, int line, const T *S) {
+    constexpr int V = line_vector<NQ, T>();
+    if constexpr (V == 1) {
+#pragma unroll
+        for (int n = 0; n < NQ; ++n) buf[slot<NQ, T>(line, n)] = S[n];
+    } else {
+        struct alignas(V * sizeof(T)) Vec { T x[V]; };
+        Vec *p = reinterpret_cast<Vec *>(buf + line * NQ);
+#pragma unroll
+        for (int n = 0; n < NQ / V; ++n) {
+            Vec v;
+#pragma unroll
+            for (int m = 0; m < V; ++m) v.x[m] = S[n * V + m];
+            p[n] = v;
+        }
+    }
+}
+
 // Sweep line `line` of buf in place.  De, Do: (Nq/2)^2 row-major; Dc[r] =
 // D[r][c] and Dcr[m] = D[c][m] for odd Nq.  The tables live in kernel
 // parameter space, so every thread reads the same constant-bank operand.
@@ -86,9 +165,10 @@ __host__ __device__ __forceinline__ void sweep_line(T *buf, int line, const Tab 
     constexpr bool ODD = (NQ & 1) != 0;
     constexpr int C = NQ / 2;
     T F[NQ];
-#pragma unroll
-    for (int n = 0; n < NQ; ++n) F[n] = buf[slot<NQ, T>(line, n)];
+    load_line<NQ, T>(buf, line, F);
     T E[HALF > 0 ? HALF : 1], O[HALF > 0 ? HALF : 1];
+    constexpr bool VEC = line_vector<NQ, T>() > 1;   // sums kept for whole-unit stores
+    T S[VEC ? NQ : 1];
 #pragma unroll
     for (int m = 0; m < HALF; ++m) {
         E[m] = F[m] + F[NQ - 1 - m];
@@ -102,9 +182,15 @@ __host__ __device__ __forceinline__ void sweep_line(T *buf, int line, const Tab 
             a = fma(tab.De[r * HALF + m], E[m], a);
             b = fma(tab.Do[r * HALF + m], O[m], b);
         }
-        buf[slot<NQ, T>(line, r)] = b + a;
-        buf[slot<NQ, T>(line, NQ - 1 - r)] = b - a;
+        if constexpr (VEC) {
+            S[r] = b + a;
+            S[NQ - 1 - r] = b - a;
+        } else {
+            buf[slot<NQ, T>(line, r)] = b + a;
+            buf[slot<NQ, T>(line, NQ - 1 - r)] = b - a;
+        }
     }
+    if constexpr (VEC) store_line<NQ, T>(buf, line, S);
     if (ODD) {
         T Sc = T(0);
 #pragma unroll

@@ -30,16 +30,28 @@ static __device__ __noinline__ double eos_pressure(double Th, const EosConstants
     return __dmul_rn(c.p0, pow(__ddiv_rn(__dmul_rn(c.R, Th), c.p0), c.gamma));
 }
 
-// p' of one point; the form is chosen per warp (see above).  Every active
-// lane of the warp must call it together.
+// The active lanes of the calling lane's group of GROUP lanes.
+template <int GROUP>
+static __device__ __forceinline__ unsigned vote_mask() {
+    unsigned lanes = __activemask();
+    if constexpr (GROUP < 32) {
+        unsigned lane;
+        asm("mov.u32 %0, %%laneid;" : "=r"(lane));
+        lanes &= ((1u << GROUP) - 1u) << (lane & ~(GROUP - 1u));
+    }
+    return lanes;
+}
+
+// p' of one point; the form is chosen per warp (see above), or per GROUP lanes.
+// Every active lane of the group must call it together.
 // Params: NativeParams or HighParams (the series coefficients c and eos).
-template <typename Params>
+template <int GROUP = 32, typename Params>
 static __device__ __forceinline__ double pressure_perturbation(double Th, double th0, double w, double A,
                                                         const Params &P) {
     const double thp = Th - th0;              // Theta'
     const double x = thp * w;                 // Theta' / Theta_ref
     const double ax = fabs(x);
-    const unsigned lanes = __activemask();
+    const unsigned lanes = vote_mask<GROUP>();
     if (__all_sync(lanes, ax <= 0.015625)) {
         double g = P.c[8];
 #pragma unroll
@@ -75,10 +87,10 @@ static __device__ __forceinline__ EosRef32 eos_reference_f32(float th0, const Pa
 }
 
 // Params: MixedParams or HighParams32 (c, K, gm1, gamma).
-template <typename Params>
+template <int GROUP = 32, typename Params>
 static __device__ __forceinline__ float pressure_perturbation_f32(float thp, float th0, EosRef32 r,
                                                            const Params &P) {
-    const unsigned lanes = __activemask();
+    const unsigned lanes = vote_mask<GROUP>();
     if (__all_sync(lanes, th0 > 0.0f)) {
         const float x = thp * r.w;
         const float ax = fabsf(x);
@@ -102,10 +114,10 @@ static __device__ __forceinline__ float pressure_perturbation_f32(float thp, flo
     return P.K * powf(thp, P.gamma);
 }
 
-template <typename Params>
+template <int GROUP = 32, typename Params>
 static __device__ __forceinline__ float pressure_perturbation_f32(float thp, float th0,
                                                            const Params &P) {
-    if (th0 > 0.0f) return pressure_perturbation_f32(thp, th0, eos_reference_f32(th0, P), P);
+    if (th0 > 0.0f) return pressure_perturbation_f32<GROUP>(thp, th0, eos_reference_f32(th0, P), P);
     return P.K * powf(thp, P.gamma);
 }
 

@@ -196,10 +196,12 @@ __host__ __device__ __forceinline__ int sweep_line_fixed(double *buf, int line, 
         return kFixNone;
     }
     long long X[NQ];
+    double F[NQ];
+    load_line<NQ, double>(buf, line, F);
     uint32_t top = 0, any = 0;
 #pragma unroll
     for (int n = 0; n < NQ; ++n) {
-        X[n] = fix_bits(buf[slot<NQ, double>(line, n)]);
+        X[n] = fix_bits(F[n]);
         const uint32_t h = (uint32_t)((unsigned long long)X[n] >> 32) & 0x7FFFFFFFu;
         top = h > top ? h : top;
         any |= (uint32_t)X[n];
@@ -214,7 +216,12 @@ __host__ __device__ __forceinline__ int sweep_line_fixed(double *buf, int line, 
     }
 #pragma unroll
     for (int n = 0; n < NQ; ++n) X[n] = fix_from_bits(X[n], e);
-    sweep_fixed<NQ>(X, ft, [&](int n, long long S) { buf[slot<NQ, double>(line, n)] = fix_double(S); });
+    if constexpr (line_vector<NQ, double>() > 1) {
+        sweep_fixed<NQ>(X, ft, [&](int n, long long S) { F[n] = fix_double(S); });
+        store_line<NQ, double>(buf, line, F);
+    } else {
+        sweep_fixed<NQ>(X, ft, [&](int n, long long S) { buf[slot<NQ, double>(line, n)] = fix_double(S); });
+    }
     return e;
 }
 

@@ -29,7 +29,8 @@
 //    N = 4, 512 elements, a call among others: 22.5 and 14.3 us.
 //  * Jinv is applied once to the sum of the three sweeps (opt. level 8).
 //
-// One CTA of Nq^3 threads per element, in three phases: fluxes by point,
+// One CTA of Nq^3 threads per element (several elements from Nq = 6 down, so
+// that a CTA has a few hundred threads: cta_elements), in three phases: fluxes by point,
 // sweeps by line (in place), combination by point.
 #include <cuda_runtime.h>
 
@@ -46,77 +47,91 @@ namespace {
 // at most 32 CTAs.
 template <int NQ>
 constexpr int min_ctas() {
-    constexpr int n = 1024 / (NQ * NQ * NQ);
+    constexpr int n = 1024 / (cta_threads<NQ>());
     return n < 1 ? 1 : (n > 32 ? 32 : n);
 }
 
 // TRACERS: nf = 5 + tracers fields (up to 8) at run time; the tracers follow
 // Theta with flux Q u_d and no source.  Without tracers nf is 5.
 template <int NQ, bool TRACERS>
-__global__ void __launch_bounds__(NQ * NQ * NQ, min_ctas<NQ>())
+__global__ void __launch_bounds__((cta_threads<NQ>()), min_ctas<NQ>())
 vol_rhs_fp64_kernel(DeviceGeometry geo, const __grid_constant__ NativeParams P,
                     FixedTables<16, 4> fix, const double *__restrict__ q, double *__restrict__ rhs, int64_t M, int64_t e0,
-                    int nf_run) {
+                    int64_t e_end, int nf_run) {
     constexpr int N3 = NQ * NQ * NQ;
     constexpr int NL = NQ * NQ;               // lines per (direction, field)
     const int nf = TRACERS ? nf_run : kFields;
-    extern __shared__ double sF[];            // [direction*nf + field][slot]
-    short *sE = reinterpret_cast<short *>(sF + 3 * nf * N3);   // [direction*nf + field][line]
+    constexpr int EPC = cta_elements<NQ>();
+    constexpr int TE = element_threads<NQ>(), NT = cta_threads<NQ>();
+    constexpr int EW = EPC * N3;              // one (direction, field) block
+    constexpr int EL = EPC * NL;              // lines of a block
+    extern __shared__ __align__(16) double sF[];   // [direction*nf + field][element][slot]
+    short *sE = reinterpret_cast<short *>(sF + 3 * nf * EW);   // [direction*nf + field][element][line]
 
     const int l = threadIdx.x;
-    const int i = l % NQ, j = (l / NQ) % NQ, k = l / (NQ * NQ);
-    const int64_t node = (e0 + blockIdx.x) * N3 + l;
+    const int el = l / TE, p = l % TE;
+    const int i = p % NQ, j = (p / NQ) % NQ, k = p / (NQ * NQ);
+    const int64_t e = e0 + blockIdx.x * (int64_t)EPC + el;
+    // threads with a point: not the padding of an element, nor past the last one
+    const bool active = EPC == 1 || (p < N3 && e < e_end);
+    const int64_t node = e * N3 + p;
 
     // ---- phase 1: p', fluxes ----------------------------------------
-    const double rho = q[node];
-    const double U[3] = {q[M + node], q[2 * M + node], q[3 * M + node]};
-    const double Th = q[4 * M + node];
-    const double pp = pressure_perturbation(Th, geo.theta_ref[node], geo.w[node], geo.A[node], P);
-    const double rinv = __drcp_rn(rho);
-    double Q[kMaxFields - kFields];
-    if constexpr (TRACERS) {
-#pragma unroll
-        for (int t = 0; t < kMaxFields - kFields; ++t)
-            Q[t] = kFields + t < nf ? q[(kFields + t) * M + node] : 0.0;
-    }
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const double g1 = geo.g[3 * d][node], g2 = geo.g[3 * d + 1][node],
-                     g3 = geo.g[3 * d + 2][node];
-        const double v = fma(g3, U[2], fma(g2, U[1], g1 * U[0]));
-        const double u = v * rinv;
-        const int s = dir_slot<NQ, double>(d, i, j, k);
-        double *F = sF + d * nf * N3 + s;
-        F[0 * N3] = v;
-        F[1 * N3] = fma(U[0], u, g1 * pp);
-        F[2 * N3] = fma(U[1], u, g2 * pp);
-        F[3 * N3] = fma(U[2], u, g3 * pp);
-        F[4 * N3] = Th * u;
+    double rho = 1.0;
+    if (active) {
+        rho = q[node];
+        const double U[3] = {q[M + node], q[2 * M + node], q[3 * M + node]};
+        const double Th = q[4 * M + node];
+        const double pp = pressure_perturbation<vote_lanes<NQ>()>(Th, geo.theta_ref[node], geo.w[node],
+                                                                  geo.A[node], P);
+        const double rinv = __drcp_rn(rho);
+        double Q[kMaxFields - kFields];
         if constexpr (TRACERS) {
 #pragma unroll
             for (int t = 0; t < kMaxFields - kFields; ++t)
-                if (kFields + t < nf) F[(kFields + t) * N3] = Q[t] * u;
+                Q[t] = kFields + t < nf ? q[(kFields + t) * M + node] : 0.0;
+        }
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const double g1 = geo.g[3 * d][node], g2 = geo.g[3 * d + 1][node],
+                         g3 = geo.g[3 * d + 2][node];
+            const double v = fma(g3, U[2], fma(g2, U[1], g1 * U[0]));
+            const double u = v * rinv;
+            double *F = sF + d * nf * EW + el * N3 + dir_slot<NQ, double>(d, i, j, k);
+            F[0 * EW] = v;
+            F[1 * EW] = fma(U[0], u, g1 * pp);
+            F[2 * EW] = fma(U[1], u, g2 * pp);
+            F[3 * EW] = fma(U[2], u, g3 * pp);
+            F[4 * EW] = Th * u;
+            if constexpr (TRACERS) {
+#pragma unroll
+                for (int t = 0; t < kMaxFields - kFields; ++t)
+                    if (kFields + t < nf) F[(kFields + t) * EW] = Q[t] * u;
+            }
         }
     }
     __syncthreads();
 
     // ---- phase 2: even-odd sweeps, one line per task, in place --------
-    for (int item = l; item < 3 * nf * NL; item += N3)
-        sE[item] = (short)sweep_line_fixed<NQ>(sF + (item / NL) * N3, item % NL, P, fix);
+    for (int item = l; item < 3 * nf * EL; item += NT)   // a block's lines are contiguous
+        sE[item] = (short)sweep_line_fixed<NQ>(sF + (item / EL) * EW, item % EL, P, fix);
     __syncthreads();
+    if (!active) return;
 
     // ---- phase 3: combine, scale, gravity, store ----------------------
     const double Jinv = geo.Jinv[node];
     const double drho = rho - geo.rho_ref[node];
+    const double *sFe = sF + el * N3;
+    const short *sEe = sE + el * NL;
 #pragma unroll
     for (int b = 0; b < (TRACERS ? kMaxFields : kFields); ++b) {
         if (TRACERS && b >= nf) break;
-        const double R = fixed_sum3<NQ>(sF[(0 * nf + b) * N3 + dir_slot<NQ, double>(0, i, j, k)],
-                                    sE[(0 * nf + b) * NL + NQ * k + j],
-                                    sF[(1 * nf + b) * N3 + dir_slot<NQ, double>(1, i, j, k)],
-                                    sE[(1 * nf + b) * NL + NQ * k + i],
-                                    sF[(2 * nf + b) * N3 + dir_slot<NQ, double>(2, i, j, k)],
-                                    sE[(2 * nf + b) * NL + NQ * j + i], fix.shift);
+        const double R = fixed_sum3<NQ>(sFe[(0 * nf + b) * EW + dir_slot<NQ, double>(0, i, j, k)],
+                                    sEe[(0 * nf + b) * EL + NQ * k + j],
+                                    sFe[(1 * nf + b) * EW + dir_slot<NQ, double>(1, i, j, k)],
+                                    sEe[(1 * nf + b) * EL + NQ * k + i],
+                                    sFe[(2 * nf + b) * EW + dir_slot<NQ, double>(2, i, j, k)],
+                                    sEe[(2 * nf + b) * EL + NQ * j + i], fix.shift);
         double v = -Jinv * R;
         if (b == 3) v = fma(-drho, P.eos.grav, v);
         rhs[b * M + node] = v;
@@ -126,15 +141,15 @@ vol_rhs_fp64_kernel(DeviceGeometry geo, const __grid_constant__ NativeParams P,
 template <int NQ, bool TRACERS>
 cudaError_t launch_kernel(ElemRange r, int nf, const DeviceGeometry &geo, const NativeParams &P,
                           const FixedTables<16, 4> &fix, const double *q, double *rhs, cudaStream_t s) {
-    constexpr int N3 = NQ * NQ * NQ;
-    const size_t smem = (sizeof(double) * N3 + sizeof(short) * NQ * NQ) * nf * 3;
+    constexpr int EPC = cta_elements<NQ>(), NT = cta_threads<NQ>();
+    const size_t smem = (sizeof(double) * NQ + sizeof(short)) * EPC * NQ * NQ * nf * 3;
     // The opt-in above 48 KB is per device; setting it on every launch keeps
     // multi-device processes correct and costs about a microsecond.
     cudaError_t e = cudaFuncSetAttribute(vol_rhs_fp64_kernel<NQ, TRACERS>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    vol_rhs_fp64_kernel<NQ, TRACERS><<<(unsigned)r.count, N3, smem, s>>>(geo, P, fix, q, rhs, r.M,
-                                                                         r.e0, nf);
+    vol_rhs_fp64_kernel<NQ, TRACERS><<<(unsigned)((r.count + EPC - 1) / EPC), NT, smem, s>>>(
+        geo, P, fix, q, rhs, r.M, r.e0, r.e0 + r.count, nf);
     return cudaGetLastError();
 }
 
