@@ -330,7 +330,9 @@ int numa_batch_autotune(numa_batch *b, void *stream);
 typedef struct {
     int tile[9];               /* elements per work item: a positive multiple of
                                   512 / Nq^3 (the elements one pass of 512
-                                  threads holds) */
+                                  threads holds).  The default, four passes, is
+                                  split finer in launches of few items until it
+                                  is set or autotuned */
     int sweep[9];              /* NUMA_SWEEP_CUDA_CORES or NUMA_SWEEP_TENSOR_TF32 */
     int ctas_per_sm;           /* CTAs per SM of the persistent grid: 1 .. 2
                                   (NUMA_MIXED) or 1 (NUMA_FP64); 0 = the most */

@@ -57,6 +57,7 @@ struct numa_batch {
     numa_sweep sweep = NUMA_SWEEP_CUDA_CORES;
     unsigned tc_mask = 0;  // orders (bit Nq) whose D sums run on the tensor cores (mixed only)
     int ctas_per_sm = 0;   // CTAs per SM of the persistent grid (0: the kernel's maximum)
+    bool tile_chosen = false;       // by the autotuner or set_config; else at most these
     bool costliest_first = false;   // work items sorted by points, largest first
     bool tmem_state = false;        // mixed, CUDA-core tiles: the state in tensor memory
     double tuned_ms = 0.0;          // last autotune: ms per step of the chosen configuration
@@ -97,6 +98,25 @@ std::vector<BatchItem> build_items(const std::vector<BatchInstance> &inst, const
             return a.count * a.nq * a.nq * a.nq > b.count * b.nq * b.nq * b.nq;
         });
     return items;
+}
+
+// A CTA takes an item through all its stages, so a launch of few items leaves
+// CTAs idle, and one of a few items per CTA ends with a ragged last round:
+// small batches, the rounds of an engine with few members left.  Measured, four
+// passes per item and this rule: one member of 7^3 elements of N = 4, ten steps,
+// mixed 272 and 90 us, FP64 4.12 ms (with FP64 sweeps) and 1.19 ms; two members
+// (N = 7, 8^3; N = 4, 10^3) mixed 423 and 310 us; 6 FP64 members of 4.6 million
+// points 36.4 and 35.0 ms; 12 mixed requests of the engine 3.50 and 3.34 ms.  4 to
+// 64 items per CTA measure the same but for the 6 members (36.4, 35.5, 35.0, 35.0
+// and 35.0 ms at 4, 8, 16, 32 and 64).
+void fit_passes(const std::vector<BatchInstance> &inst, int slots, const int *cap, int *mult) {
+    int64_t passes = 0;
+    for (const auto &I : inst) {
+        const int64_t ne = I.M / ((int64_t)I.nq * I.nq * I.nq), epp = elements_per_pass(I.nq);
+        passes += (ne + epp - 1) / epp;
+    }
+    const int64_t most = std::max<int64_t>(1, passes / ((int64_t)kItemsPerCta * std::max(1, slots)));
+    for (int nq = 0; nq < 9; ++nq) mult[nq] = (int)std::min<int64_t>(cap[nq], most);
 }
 
 }  // namespace numa
@@ -230,8 +250,15 @@ int numa_batch_advance(numa_batch *b, int nsteps, double dt, void *stream) {
     cudaError_t e = cudaSuccess;
     if (b->dirty) {
         drop_graph(b);
-        e = upload(b, b->inst, numa::build_items(b->inst, b->tile_mult, b->costliest_first),
-                   b->cap_stream);
+        int mult[9];
+        std::copy(b->tile_mult, b->tile_mult + 9, mult);
+        if (!b->tile_chosen)
+            numa::fit_passes(b->inst,
+                             b->num_sms * numa::batch_ctas_per_sm(b->prec == NUMA_MIXED,
+                                                                  has_tracers(b->inst),
+                                                                  b->ctas_per_sm),
+                             b->tile_mult, mult);
+        e = upload(b, b->inst, numa::build_items(b->inst, mult, b->costliest_first), b->cap_stream);
         if (e != cudaSuccess) return bfail_cuda(e, "numa_batch_advance: upload of the work list");
         b->dirty = false;
     }
@@ -418,6 +445,7 @@ int numa_batch_autotune(numa_batch *b, void *stream) {
     if (t1) cudaEventDestroy(t1);
     if (e != cudaSuccess) return bfail_cuda(e, "numa_batch_autotune");
     std::copy(cur.mult, cur.mult + 9, b->tile_mult);
+    b->tile_chosen = true;
     b->tc_mask = cur.mask;
     b->ctas_per_sm = cur.ctas;
     b->costliest_first = cur.costliest;
@@ -467,7 +495,10 @@ int numa_batch_set_config(numa_batch *b, const numa_batch_config *c) {
             return bfail(NUMA_EINVAL, "numa_batch_set_config: a sweep is not CUDA_CORES or TENSOR_TF32");
         }
     }
-    for (int nq = 2; nq <= 8; ++nq) b->tile_mult[nq] = mult[nq];
+    for (int nq = 2; nq <= 8; ++nq) {
+        b->tile_chosen = b->tile_chosen || b->tile_mult[nq] != mult[nq];
+        b->tile_mult[nq] = mult[nq];
+    }
     b->tc_mask = mask;
     b->ctas_per_sm = c->ctas_per_sm;
     if (c->state_in_tmem && !mixed)

@@ -213,18 +213,23 @@ cudaError_t prepare_batch_lsrk() {
 // FP64 has one grid (two CTAs per SM, one in the tracer form): its setting is 1.
 int batch_max_ctas_per_sm(bool mixed) { return mixed ? 2 : 1; }
 
+int batch_ctas_per_sm(bool mixed, bool tracers, int ctas_per_sm) {
+    if (!mixed) return tracers ? tile_ctas_per_sm<false, true>() : tile_ctas_per_sm<false>();
+    const int kmax = batch_max_ctas_per_sm(true);
+    return ctas_per_sm > 0 && ctas_per_sm < kmax ? ctas_per_sm : kmax;
+}
+
 cudaError_t launch_batch_lsrk(bool mixed, const BatchInstance *inst, const BatchItem *items,
                               int num_items, int *counter, const LsrkCoef &co, int nsteps,
                               double dt, int num_sms, cudaStream_t s, unsigned tc_mask,
                               int ctas_per_sm, bool tmem_state, bool tracers) {
     if (num_items <= 0 || nsteps <= 0) return cudaSuccess;
-    const int kmax = batch_max_ctas_per_sm(mixed);
-    const int k = ctas_per_sm > 0 && ctas_per_sm < kmax ? ctas_per_sm : kmax;
+    const int k = batch_ctas_per_sm(mixed, tracers, ctas_per_sm);
     if (tracers && mixed)   // the shared-memory-state tile's tracer form
         batch_lsrk_kernel<true, true><<<num_sms * k, kThreads, tile_smem_bytes<true, true>(), s>>>(
             inst, items, num_items, counter, co, nsteps, dt);
     else if (tracers)
-        batch_lsrk_kernel<false, true><<<num_sms * tile_ctas_per_sm<false, true>(), kThreads, tile_smem_bytes<false, true>(), s>>>(
+        batch_lsrk_kernel<false, true><<<num_sms * k, kThreads, tile_smem_bytes<false, true>(), s>>>(
             inst, items, num_items, counter, co, nsteps, dt);
     else if (mixed && (tc_mask != 0 || tmem_state))
         batch_lsrk_tc_kernel<<<num_sms * k, kThreads, kTcSmemBytes, s>>>(
@@ -233,7 +238,7 @@ cudaError_t launch_batch_lsrk(bool mixed, const BatchInstance *inst, const Batch
         batch_lsrk_kernel<true><<<num_sms * k, kThreads, tile_smem_bytes<true>(), s>>>(
             inst, items, num_items, counter, co, nsteps, dt);
     else
-        batch_lsrk_kernel<false><<<num_sms * tile_ctas_per_sm<false>(), kThreads, tile_smem_bytes<false>(), s>>>(
+        batch_lsrk_kernel<false><<<num_sms * k, kThreads, tile_smem_bytes<false>(), s>>>(
             inst, items, num_items, counter, co, nsteps, dt);
     return cudaGetLastError();
 }

@@ -247,6 +247,10 @@ int numa_engine_create(numa_precision prec, size_t budget_bytes, int max_members
     cudaError_t err = cudaGetDevice(&e->device);
     if (err == cudaSuccess)
         err = cudaDeviceGetAttribute(&e->num_sms, cudaDevAttrMultiProcessorCount, e->device);
+    // Fewer passes per item in small launches (fit_passes): below tile_mult
+    // passes the items are fewer than 2 kItemsPerCta per resident CTA, and one
+    // partial item per member.
+    e->items_cap += 2 * (size_t)numa::kItemsPerCta * 2 * (size_t)e->num_sms;
     if (err == cudaSuccess) err = numa::prepare_batch_lsrk();
     if (err == cudaSuccess) err = cudaMalloc(&e->d_arena, budget_bytes);
     for (auto &sl : e->slot) {
@@ -460,7 +464,10 @@ int numa_engine_progress(numa_engine *e, int64_t *done_ids, int max_done, int *n
             e->point_stages += 5.0 * I.nsteps * (double)r.mesh->M;
         }
         int mult[9];
-        std::fill(mult, mult + 9, e->tile_mult);
+        int cap[9];
+        std::fill(cap, cap + 9, e->tile_mult);
+        numa::fit_passes(inst, e->num_sms * numa::batch_ctas_per_sm(e->prec == NUMA_MIXED, tracers, 0),
+                         cap, mult);
         std::vector<numa::BatchItem> items = numa::build_items(inst, mult);
         if (per_member) {
             // costliest items first (points x steps), so that the long ones

@@ -133,9 +133,17 @@ cudaError_t launch_batch_lsrk(bool mixed, const BatchInstance *inst, const Batch
                               int ctas_per_sm = 0, bool tmem_state = false,
                               bool tracers = false);
 int batch_max_ctas_per_sm(bool mixed);
+// CTAs per SM of a launch with these settings.
+int batch_ctas_per_sm(bool mixed, bool tracers, int ctas_per_sm);
 
 // Elements one CTA pass holds for order Nq (512 threads, one per point).
 inline int elements_per_pass(int nq) { return 512 / (nq * nq * nq); }
+
+// Passes per work item of a launch over `slots` resident CTAs: cap[nq] or, where
+// that leaves fewer than kItemsPerCta items per CTA, as many as give that
+// number, at least one (batch_abi.cu).
+constexpr int kItemsPerCta = 16;
+void fit_passes(const std::vector<BatchInstance> &inst, int slots, const int *cap, int *mult);
 
 // Work list for instances with tile_mult[nq] passes per item (batch_abi.cu);
 // costliest_first: items sorted by points, largest first (stable).
