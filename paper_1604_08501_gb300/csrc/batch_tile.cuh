@@ -253,7 +253,7 @@ __device__ void run_tile(const BatchInstance &I, int64_t e0, int64_t count,
                     if constexpr (MIXED)
                         rinv = __frcp_rn(rho);   // the correctly rounded 1/rho, as 1.0f / rho
                     else
-                        rinv = __drcp_rn(rho);   // the correctly rounded 1/rho, as 1.0 / rho
+                        rinv = rcp_fp64(rho);
 #pragma unroll
                     for (int d = 0; d < 3; ++d) {
                         const T g1 = g[3 * d], g2 = g[3 * d + 1], g3 = g[3 * d + 2];
@@ -297,16 +297,26 @@ __device__ void run_tile(const BatchInstance &I, int64_t e0, int64_t count,
                 }
                 __syncthreads();
                 // ---- phase 3: rhs, stage update ------------------------
-                // the sum of field b's three sweeps at the thread's point
-                auto sum3 = [&](int b) -> T {
-                    const T r = sF[f[0] + b * BLK], s = sF[f[1] + b * BLK], t = sF[f[2] + b * BLK];
+                // -J^-1 times the sums of fields b0 .. of the three sweeps at the
+                // thread's point
+                auto sums = [&](auto &v, int b0, T jinv) {
+                    constexpr int NB = sizeof(v) / sizeof(T);
                     if constexpr (MIXED) {
-                        return r + s + t;
+#pragma unroll
+                        for (int b = 0; b < NB; ++b) {
+                            const int o = (b0 + b) * BLK;
+                            v[b] = -jinv * (sF[f[0] + o] + sF[f[1] + o] + sF[f[2] + o]);
+                        }
                     } else {
                         constexpr int EB = EPP * NL;   // lines of one (direction, field)
-                        const short *E = sE + b * EB + el * NL;
-                        return fixed_sum3<NQ>(r, E[NQ * k + j], s, E[NF * EB + NQ * k + i], t,
-                                              E[2 * NF * EB + NQ * j + i], c_fixed[NQ].shift);
+                        const short *E = sE + b0 * EB + el * NL;
+                        fixed_sums<NQ>(
+                            v, c_fixed[NQ].shift, jinv,
+                            [&](int d, int b) { return sF[f[d] + (b0 + b) * BLK]; },
+                            [&](int d, int b) {
+                                return (int)E[(d * NF + b) * EB +
+                                              (d == 0 ? NQ * k + j : d == 1 ? NQ * k + i : NQ * j + i)];
+                            });
                     }
                 };
                 if (active) {
@@ -319,10 +329,11 @@ __device__ void run_tile(const BatchInstance &I, int64_t e0, int64_t count,
                         jinv = jinv_g;
                         drho = Q(0) - rho_ref_g;
                     }
+                    T v[kFields];
+                    sums(v, 0, jinv);
 #pragma unroll
                     for (int b = 0; b < kFields; ++b) {
-                        const T R = sum3(b);
-                        T rhs = -jinv * R;
+                        T rhs = v[b];
                         if (b == 3) rhs = fma(-drho, grav, rhs);
                         const T d = fma(a, DQ(b), dtt * rhs);
                         DQ(b) = d;
@@ -333,8 +344,9 @@ __device__ void run_tile(const BatchInstance &I, int64_t e0, int64_t count,
                         for (int t = 0; t < NTR; ++t) {
                             if (kFields + t >= nf) break;
                             const int b = kFields + t;
-                            const T R = sum3(b);
-                            const T d = fma(a, DQT(t), dtt * (-jinv * R));
+                            T w[1];
+                            sums(w, b, jinv);
+                            const T d = fma(a, DQT(t), dtt * w[0]);
                             DQT(t) = d;
                             QT(t) = fma(bcoef, d, QT(t));
                         }

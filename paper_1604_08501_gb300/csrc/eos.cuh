@@ -8,7 +8,9 @@
 // difference of two pressures, without its cancellation.
 //
 // FP64 has three forms, each accurate to a few ulps over its whole range:
-// the series to 9 terms for |x| <= 1/64 and to 15 terms for |x| <= 1/8
+// the series to 9 terms for |x| <= 1/64 (the last four in FP32 where they are
+// below 2^-34 of the sum, as for any gamma near 1.4: FP32's error is then below
+// 2^-58 of it) and to 15 terms for |x| <= 1/8
 // (truncation below 2^-55 relative for gamma near 1.4), and
 // p_ref expm1(gamma log1p(x)) for any x > -1.  A warp takes the widest form
 // any of its lanes needs, so that a warp never runs several of them one after
@@ -19,6 +21,7 @@
 // below 2^-26), expm1f(gamma log1pf(x)) beyond, chosen per warp.
 #pragma once
 
+#include "fp64_ops.cuh"
 #include "kernel_params.h"
 
 namespace numa {
@@ -50,15 +53,29 @@ static __device__ __forceinline__ double pressure_perturbation(double Th, double
                                                         const Params &P) {
     const double thp = Th - th0;              // Theta'
     const double x = thp * w;                 // Theta' / Theta_ref
+    // |x| compared as bits, on the integer pipe (a NaN's are larger)
+    const long long xb = __double_as_longlong(x);
+    const unsigned long long ab = (unsigned long long)xb & 0x7FFFFFFFFFFFFFFFull;
     const double ax = fabs(x);
     const unsigned lanes = vote_mask<GROUP>();
-    if (__all_sync(lanes, ax <= 0.015625)) {
-        double g = P.c[8];
+    if (__all_sync(lanes, ab <= 0x3F90000000000000ull)) {   // 1/64
+        double g;
+        if (P.tail_f32) {   // uniform
+            const float xf = f64_to_f32_trunc(xb);
+            float t = P.ct[3];
 #pragma unroll
-        for (int k = 7; k >= 0; --k) g = fma(g, x, P.c[k]);   // sum_k c_{k+1} x^k
+            for (int k = 2; k >= 0; --k) t = fmaf(t, xf, P.ct[k]);
+            g = f32_to_f64(t);
+        } else {
+            g = P.c[8];
+#pragma unroll
+            for (int k = 7; k >= 5; --k) g = fma(g, x, P.c[k]);
+        }
+#pragma unroll
+        for (int k = 4; k >= 0; --k) g = fma(g, x, P.c[k]);   // sum_k c_{k+1} x^k
         return (A * thp) * g;
     }
-    if (__all_sync(lanes, ax <= 0.125)) {
+    if (__all_sync(lanes, ab <= 0x3FC0000000000000ull)) {   // 1/8
         double g = P.c[14];
 #pragma unroll
         for (int k = 13; k >= 0; --k) g = fma(g, x, P.c[k]);

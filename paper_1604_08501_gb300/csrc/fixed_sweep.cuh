@@ -20,11 +20,12 @@
 //    dropped.  Three multiply-adds per product.
 //  * S_i = a_i + b_i and S_{N-i} = b_i - a_i, |S| <= 2^60, replace the line's
 //    fluxes; the value is S 2^(e - 1024 - s).  Phase 3 adds a point's three sums
-//    as integers at the largest of their exponents (|sum| <= 3 2^60) and rounds
-//    once to FP64.
+//    as integers at the largest of their exponents (|sum| <= 3 2^60), multiplies
+//    them by J^-1 as integers and rounds once to FP64 (fixed_sums).
 //
 // Measured: vol_rhs_fp64_kernel at N = 7, 32768 elements, 4.949 -> 1.881 ms; the
-// FP64 batch 2.07 times as fast.
+// FP64 batch 2.07 times as fast.  (Rounded before an FP64 multiply by J^-1, one
+// test for each field; all fields' integer chains side by side: see vol_fp64.cu.)
 //
 // Error: at most 1 in each X and 2^-1 in each integer D entry, so at most
 // 2^-55 (largest |D| row sum) (largest flux of the line), as a bound; the
@@ -123,6 +124,40 @@ __host__ __device__ __forceinline__ double fix_to_double(long long R, int e, int
     const int E = e - shift + 61 - lz;
     const unsigned long long v = ((unsigned long long)(uint32_t)E << 52) + (m >> 11) + ((m >> 10) & 1ull);
     return a == 0ull ? 0.0 : fix_double((long long)(v | ((unsigned long long)s & (1ull << 63))));
+}
+
+__host__ __device__ __forceinline__ unsigned long long fix_mulhi(unsigned long long a,
+                                                                 unsigned long long b) {
+#ifdef __CUDA_ARCH__
+    return __umul64hi(a, b);
+#else
+    return (unsigned long long)(((unsigned __int128)a * b) >> 64);
+#endif
+}
+
+// -y R 2^(e - 1024 - s), rounded once (to nearest, ties away from zero): the
+// integer's leading 64 bits times the 53 of y (exponent field ey), a multiply
+// on the integer pipes.  ok is cleared where the product is not a normal number.
+__host__ __device__ __forceinline__ double fix_scale(long long R, int e, int shift, double y, int ey,
+                                                     bool &ok) {
+    const long long yb = fix_bits(y);
+    const long long s = R >> 63;
+    const unsigned long long a = (unsigned long long)((R ^ s) - s);
+    const int lz = fix_clz(a);
+    // y's mantissa with its hidden bit at 63; the product in [2^62, 2^64)
+    const unsigned long long my = ((unsigned long long)yb << 11) | (1ull << 63);
+    unsigned long long p = fix_mulhi(a << (lz & 63), my);
+    const int up = (long long)p < 0 ? 0 : 1;
+    p <<= up;
+    // exponent field of 2^(63 - lz) 2^(e - 1024 - s) y, less the hidden bit's one
+    const int E = e - shift + 61 - lz + ey - 1023 + 1 - up;
+    const unsigned long long v = ((unsigned long long)(uint32_t)E << 52) + (p >> 11) + ((p >> 10) & 1ull);
+    ok = ok && (a == 0ull || (unsigned)(E - 1) < 2044u);
+    return a == 0ull ? 0.0
+                     : fix_double((long long)(v | ((unsigned long long)(~(s ^ yb)) & (1ull << 63))));
+}
+__host__ __device__ __forceinline__ int fix_exponent(double y) {
+    return (int)((unsigned long long)fix_bits(y) >> 52) & 0x7FF;
 }
 
 // The FP64 sweep, for the lines that cannot be fixed point.  Out of line: its
@@ -225,27 +260,43 @@ __host__ __device__ __forceinline__ int sweep_line_fixed(double *buf, int line, 
     return e;
 }
 
-// The sum of a point's three directions where a line is in FP64 (rare).
-static __host__ __device__ __attribute__((noinline)) double fixed_sum3_slow(double r, int er, double s, int es, double t,
-                                                      int et, int shift) {
+// -y times the sum of a point's three directions where a line is in FP64, or
+// the integer multiply does not take y (rare).
+static __host__ __device__ __attribute__((noinline)) double fixed_sum3_slow(double r, int er, double s,
+                                                                            int es, double t, int et,
+                                                                            int shift, double y) {
     const double R = er < 0 ? r : fix_to_double(fix_bits(r), er, shift);
     const double S = es < 0 ? s : fix_to_double(fix_bits(s), es, shift);
     const double T = et < 0 ? t : fix_to_double(fix_bits(t), et, shift);
-    return R + S + T;
+    return -y * (R + S + T);
 }
 
-// The sum of a point's three directions, from the slots' bits (r, s, t) and
-// the lines' exponents.
-template <int NQ>
-__host__ __device__ __forceinline__ double fixed_sum3(double r, int er, double s, int es, double t,
-                                                      int et, int shift) {
-    if constexpr (!fixed_point<NQ>()) return r + s + t;
-    if ((er | es | et) < 0) return fixed_sum3_slow(r, er, s, es, t, et, shift);
-    const int m = er > es ? er : es, e = m > et ? m : et;
-    const long long R = fix_shr(fix_bits(r), e - er) +
-                        fix_shr(fix_bits(s), e - es) +
-                        fix_shr(fix_bits(t), e - et);
-    return fix_to_double(R, e, shift);
+// v[b] = -y times the sum of a point's three directions, b < NB: at(d, b) gives
+// the slot's bits and ex(d, b) the line's exponent.  One test for all of them,
+// after the integer operations, so that their chains run side by side.
+template <int NQ, int NB, typename At, typename Ex>
+__host__ __device__ __forceinline__ void fixed_sums(double (&v)[NB], int shift, double y, At at, Ex ex) {
+    if constexpr (!fixed_point<NQ>()) {
+#pragma unroll
+        for (int b = 0; b < NB; ++b) v[b] = -y * (at(0, b) + at(1, b) + at(2, b));
+        return;
+    }
+    const int ey = fix_exponent(y);
+    bool ok = (unsigned)(ey - 1) < 2046u;   // not zero, subnormal, infinite or NaN
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+        const int e0 = ex(0, b), e1 = ex(1, b), e2 = ex(2, b);
+        ok = ok && (e0 | e1 | e2) >= 0;
+        const int m = e0 > e1 ? e0 : e1, e = m > e2 ? m : e2;
+        const long long R = fix_shr(fix_bits(at(0, b)), e - e0) + fix_shr(fix_bits(at(1, b)), e - e1) +
+                            fix_shr(fix_bits(at(2, b)), e - e2);
+        v[b] = fix_scale(R, e, shift, y, ey, ok);
+    }
+    if (!ok) {
+#pragma unroll
+        for (int b = 0; b < NB; ++b)
+            v[b] = fixed_sum3_slow(at(0, b), ex(0, b), at(1, b), ex(1, b), at(2, b), ex(2, b), shift, y);
+    }
 }
 
 }  // namespace numa

@@ -54,6 +54,8 @@ struct FixedTables {
 struct NativeParams {
     EosConstants eos;
     double c[15];
+    float ct[4];     // c[5..8] in FP32
+    int tail_f32;    // their share of the series is small enough for FP32
     double De[16], Do[16], Dc[4], Dcr[4];
 };
 
@@ -62,6 +64,8 @@ struct NativeParams {
 struct HighParams {
     EosConstants eos;
     double c[15];
+    float ct[4];     // c[5..8] in FP32
+    int tail_f32;    // their share of the series is small enough for FP32
     double De[64], Do[64], Dc[8], Dcr[8];
     FixedTables<64, 8> fix;
 };

@@ -135,12 +135,21 @@ void build_params(numa_vol *h, const double *D) {
     binomial_coefficients(h->eos.gamma, c);
     h->nparams.eos = h->eos;
     for (int k = 0; k < 15; ++k) h->nparams.c[k] = static_cast<double>(c[k + 1]);
+    // c_6 .. c_9 in FP32 where their share of the series at |x| <= 1/64 is below 2^-34
+    long double tail = 0.0L;
+    for (int k = 6; k <= 9; ++k) {
+        h->nparams.ct[k - 6] = static_cast<float>(c[k]);
+        tail += std::fabs(std::ldexp(c[k], -6 * (k - 1)));
+    }
+    h->nparams.tail_f32 = tail <= std::ldexp((long double)c[1], -34) ? 1 : 0;
     const long double g = h->eos.gamma;
     const float K = static_cast<float>(std::pow((long double)h->eos.p0, 1.0L - g) *
                                        std::pow((long double)h->eos.R, g));
     if (h->N >= 8) {   // the high-order kernels' parameters (FP64 and mixed)
         h->hparams.eos = h->eos;
         for (int k = 0; k < 15; ++k) h->hparams.c[k] = h->nparams.c[k];
+        for (int k = 0; k < 4; ++k) h->hparams.ct[k] = h->nparams.ct[k];
+        h->hparams.tail_f32 = h->nparams.tail_f32;
         numa::sweep_tables(h->N, D, h->hparams.De, h->hparams.Do, h->hparams.Dc, h->hparams.Dcr);
         numa::fixed_tables(h->N, D, &h->hparams.fix);
         numa::HighParams32 &m = h->hmparams;

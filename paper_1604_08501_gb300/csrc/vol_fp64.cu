@@ -27,7 +27,14 @@
 //    of the other.  Measured at N = 7, 32768 elements: 4.949 ms with FP64
 //    sweeps, 1.881 ms (59 FP64 operations' time per point) in fixed point;
 //    N = 4, 512 elements, a call among others: 22.5 and 14.3 us.
-//  * Jinv is applied once to the sum of the three sweeps (opt. level 8).
+//  * Jinv is applied once to the sum of the three sweeps (opt. level 8), as an
+//    integer multiply before the one rounding to FP64; the last terms of the
+//    pressure series are FP32 and 1/rho starts from an FP32 reciprocal
+//    (fp64_ops.cuh).  That leaves 47 of 59 FP64 operations per point: 3.5
+//    million points N = 3 383 -> 325 us, N = 4 397 -> 332 us, N = 5 394 -> 334 us;
+//    N = 7 needed smaller CTAs as well (vol_rhs_fp64_eight_kernel): 32768
+//    elements 1.881 -> 1.656 ms, the FP64 pipe 76 % busy of the 83 % that a loop of
+//    DFMAs reaches.
 //
 // One CTA of Nq^3 threads per element (several elements from Nq = 6 down, so
 // that a CTA has a few hundred threads: cta_elements), in three phases: fluxes by point,
@@ -51,13 +58,55 @@ constexpr int min_ctas() {
     return n < 1 ? 1 : (n > 32 ? 32 : n);
 }
 
+// Fluxes of one point: put(d, b, F) takes F_d[b].  Called by every active lane of
+// a vote group together (the form of the equation of state).
+template <int NQ, bool TRACERS, typename Put>
+__device__ __forceinline__ void point_fluxes(const DeviceGeometry &geo, const NativeParams &P,
+                                             const double *__restrict__ q, int64_t M, int64_t node,
+                                             int nf, Put put) {
+    const double rho = q[node];
+    const double U[3] = {q[M + node], q[2 * M + node], q[3 * M + node]};
+    const double Th = q[4 * M + node];
+    const double pp = pressure_perturbation<vote_lanes<NQ>()>(Th, geo.theta_ref[node], geo.w[node],
+                                                              geo.A[node], P);
+    const double rinv = rcp_fp64(rho);
+    double Q[kMaxFields - kFields];
+    if constexpr (TRACERS) {
+#pragma unroll
+        for (int t = 0; t < kMaxFields - kFields; ++t)
+            Q[t] = kFields + t < nf ? q[(kFields + t) * M + node] : 0.0;
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const double g1 = geo.g[3 * d][node], g2 = geo.g[3 * d + 1][node], g3 = geo.g[3 * d + 2][node];
+        const double v = fma(g3, U[2], fma(g2, U[1], g1 * U[0]));
+        const double u = v * rinv;
+        put(d, 0, v);
+        put(d, 1, fma(U[0], u, g1 * pp));
+        put(d, 2, fma(U[1], u, g2 * pp));
+        put(d, 3, fma(U[2], u, g3 * pp));
+        put(d, 4, Th * u);
+        if constexpr (TRACERS) {
+#pragma unroll
+            for (int t = 0; t < kMaxFields - kFields; ++t)
+                if (kFields + t < nf) put(d, kFields + t, Q[t] * u);
+        }
+    }
+}
+
+// Line of point (i, j, k) in direction d (the numbering of dir_slot).
+template <int NQ>
+__device__ __forceinline__ int dir_line(int d, int i, int j, int k) {
+    return d == 0 ? NQ * k + j : d == 1 ? NQ * k + i : NQ * j + i;
+}
+
 // TRACERS: nf = 5 + tracers fields (up to 8) at run time; the tracers follow
 // Theta with flux Q u_d and no source.  Without tracers nf is 5.
 template <int NQ, bool TRACERS>
 __global__ void __launch_bounds__((cta_threads<NQ>()), min_ctas<NQ>())
 vol_rhs_fp64_kernel(DeviceGeometry geo, const __grid_constant__ NativeParams P,
-                    FixedTables<16, 4> fix, const double *__restrict__ q, double *__restrict__ rhs, int64_t M, int64_t e0,
-                    int64_t e_end, int nf_run) {
+                    FixedTables<16, 4> fix, const double *__restrict__ q,
+                    double *__restrict__ rhs, int64_t M, int64_t e0, int64_t e_end, int nf_run) {
     constexpr int N3 = NQ * NQ * NQ;
     constexpr int NL = NQ * NQ;               // lines per (direction, field)
     const int nf = TRACERS ? nf_run : kFields;
@@ -77,38 +126,12 @@ vol_rhs_fp64_kernel(DeviceGeometry geo, const __grid_constant__ NativeParams P,
     const int64_t node = e * N3 + p;
 
     // ---- phase 1: p', fluxes ----------------------------------------
-    double rho = 1.0;
     if (active) {
-        rho = q[node];
-        const double U[3] = {q[M + node], q[2 * M + node], q[3 * M + node]};
-        const double Th = q[4 * M + node];
-        const double pp = pressure_perturbation<vote_lanes<NQ>()>(Th, geo.theta_ref[node], geo.w[node],
-                                                                  geo.A[node], P);
-        const double rinv = __drcp_rn(rho);
-        double Q[kMaxFields - kFields];
-        if constexpr (TRACERS) {
+        int sl[3];
 #pragma unroll
-            for (int t = 0; t < kMaxFields - kFields; ++t)
-                Q[t] = kFields + t < nf ? q[(kFields + t) * M + node] : 0.0;
-        }
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const double g1 = geo.g[3 * d][node], g2 = geo.g[3 * d + 1][node],
-                         g3 = geo.g[3 * d + 2][node];
-            const double v = fma(g3, U[2], fma(g2, U[1], g1 * U[0]));
-            const double u = v * rinv;
-            double *F = sF + d * nf * EW + el * N3 + dir_slot<NQ, double>(d, i, j, k);
-            F[0 * EW] = v;
-            F[1 * EW] = fma(U[0], u, g1 * pp);
-            F[2 * EW] = fma(U[1], u, g2 * pp);
-            F[3 * EW] = fma(U[2], u, g3 * pp);
-            F[4 * EW] = Th * u;
-            if constexpr (TRACERS) {
-#pragma unroll
-                for (int t = 0; t < kMaxFields - kFields; ++t)
-                    if (kFields + t < nf) F[(kFields + t) * EW] = Q[t] * u;
-            }
-        }
+        for (int d = 0; d < 3; ++d) sl[d] = d * nf * EW + el * N3 + dir_slot<NQ, double>(d, i, j, k);
+        point_fluxes<NQ, TRACERS>(geo, P, q, M, node, nf,
+                                  [&](int d, int b, double F) { sF[sl[d] + b * EW] = F; });
     }
     __syncthreads();
 
@@ -120,21 +143,121 @@ vol_rhs_fp64_kernel(DeviceGeometry geo, const __grid_constant__ NativeParams P,
 
     // ---- phase 3: combine, scale, gravity, store ----------------------
     const double Jinv = geo.Jinv[node];
-    const double drho = rho - geo.rho_ref[node];
-    const double *sFe = sF + el * N3;
-    const short *sEe = sE + el * NL;
+    const double drho = q[node] - geo.rho_ref[node];
+    int sl[3], ln[3];
 #pragma unroll
-    for (int b = 0; b < (TRACERS ? kMaxFields : kFields); ++b) {
-        if (TRACERS && b >= nf) break;
-        const double R = fixed_sum3<NQ>(sFe[(0 * nf + b) * EW + dir_slot<NQ, double>(0, i, j, k)],
-                                    sEe[(0 * nf + b) * EL + NQ * k + j],
-                                    sFe[(1 * nf + b) * EW + dir_slot<NQ, double>(1, i, j, k)],
-                                    sEe[(1 * nf + b) * EL + NQ * k + i],
-                                    sFe[(2 * nf + b) * EW + dir_slot<NQ, double>(2, i, j, k)],
-                                    sEe[(2 * nf + b) * EL + NQ * j + i], fix.shift);
-        double v = -Jinv * R;
-        if (b == 3) v = fma(-drho, P.eos.grav, v);
-        rhs[b * M + node] = v;
+    for (int d = 0; d < 3; ++d) {
+        sl[d] = d * nf * EW + el * N3 + dir_slot<NQ, double>(d, i, j, k);
+        ln[d] = d * nf * EL + el * NL + dir_line<NQ>(d, i, j, k);
+    }
+    double v[kFields];
+    fixed_sums<NQ>(v, fix.shift, Jinv, [&](int d, int b) { return sF[sl[d] + b * EW]; },
+                   [&](int d, int b) { return (int)sE[ln[d] + b * EL]; });
+    v[3] = fma(-drho, P.eos.grav, v[3]);
+#pragma unroll
+    for (int b = 0; b < kFields; ++b) rhs[b * M + node] = v[b];
+    if constexpr (TRACERS) {
+#pragma unroll
+        for (int b = kFields; b < kMaxFields; ++b) {
+            if (b >= nf) break;
+            double w[1];
+            fixed_sums<NQ>(w, fix.shift, Jinv, [&](int d, int) { return sF[sl[d] + b * EW]; },
+                           [&](int d, int) { return (int)sE[ln[d] + b * EL]; });
+            rhs[b * M + node] = w[0];
+        }
+    }
+}
+
+// N = 7 without tracers: 256 threads per element, two points each, so that four
+// CTAs share an SM and more phases mix (two of 512 threads left the FP64 pipe
+// idle a third of the time once the integer phases had become as long as the
+// FP64 one).  Four CTAs leave 57 KB of shared memory each, 13 of an element's
+// 15 flux blocks: the t fluxes of rho and Theta wait in their own outputs' place
+// in rhs, which nothing else reads or writes meanwhile, until the sums of the
+// momenta are done; they then take two of the momenta's blocks.  Measured, 6912
+// elements: two CTAs of 512 threads 425 us, three of 256 405 us, three of 320
+// 441 us (registers), this 365 us.
+constexpr int kEight = 8, kEightThreads = 256, kEightBlocks = 13;
+constexpr size_t kEightSmem = kEightBlocks * (sizeof(double) * 512 + sizeof(short) * 64);
+
+// Block of direction d and field b: 5 d + b for r and s; t: the momenta's 10, 11, 12.
+__device__ __forceinline__ constexpr int eight_block(int d, int b) { return d < 2 ? 5 * d + b : 9 + b; }
+
+__global__ void __launch_bounds__(kEightThreads, 4)
+vol_rhs_fp64_eight_kernel(DeviceGeometry geo, const __grid_constant__ NativeParams P,
+                          FixedTables<16, 4> fix, const double *__restrict__ q, double *rhs,
+                          int64_t M, int64_t e0) {
+    constexpr int NQ = kEight, N3 = 512, NL = 64, NT = kEightThreads;
+    extern __shared__ __align__(16) double sF[];                       // [block][slot]
+    short *sE = reinterpret_cast<short *>(sF + kEightBlocks * N3);     // [block][line]
+    const int l = threadIdx.x;
+    const int i = l % NQ, j = (l / NQ) % NQ, k0 = l / NL;   // points (i, j, k0) and (i, j, k0 + 4)
+    const int64_t node0 = (e0 + blockIdx.x) * N3 + l;
+
+    // ---- phase 1: p', fluxes ----------------------------------------
+#pragma unroll 1
+    for (int x = 0; x < 2; ++x) {
+        const int k = k0 + 4 * x;
+        const int64_t node = node0 + x * NT;
+        int sl[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) sl[d] = dir_slot<NQ, double>(d, i, j, k);
+        point_fluxes<NQ, false>(geo, P, q, M, node, kFields, [&](int d, int b, double F) {
+            if (d == 2 && (b == 0 || b == 4)) rhs[b * M + node] = F;
+            else sF[eight_block(d, b) * N3 + sl[d]] = F;
+        });
+    }
+    __syncthreads();
+    // ---- phase 2: the sweeps of the 13 blocks, one line per task -----------
+#pragma unroll 1
+    for (int item = l; item < kEightBlocks * NL; item += NT)
+        sE[item] = (short)sweep_line_fixed<NQ>(sF + (item / NL) * N3, item % NL, P, fix);
+    __syncthreads();
+    // ---- phase 3: the momenta; the waiting fluxes into blocks 10 and 11, whose
+    // slots of these points this thread alone has read
+#pragma unroll 1
+    for (int x = 0; x < 2; ++x) {
+        const int k = k0 + 4 * x;
+        const int64_t node = node0 + x * NT;
+        int sl[3], ln[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            sl[d] = dir_slot<NQ, double>(d, i, j, k);
+            ln[d] = dir_line<NQ>(d, i, j, k);
+        }
+        const double f0 = rhs[node], f4 = rhs[4 * M + node];
+        const double drho = q[node] - geo.rho_ref[node];
+        double v[3];
+        fixed_sums<NQ>(v, fix.shift, geo.Jinv[node],
+                       [&](int d, int b) { return sF[eight_block(d, b + 1) * N3 + sl[d]]; },
+                       [&](int d, int b) { return (int)sE[eight_block(d, b + 1) * NL + ln[d]]; });
+        rhs[M + node] = v[0];
+        rhs[2 * M + node] = v[1];
+        rhs[3 * M + node] = fma(-drho, P.eos.grav, v[2]);
+        sF[10 * N3 + sl[2]] = f0;
+        sF[11 * N3 + sl[2]] = f4;
+    }
+    __syncthreads();
+    if (l < 2 * NL)
+        sE[10 * NL + l] = (short)sweep_line_fixed<NQ>(sF + (10 + l / NL) * N3, l % NL, P, fix);
+    __syncthreads();
+    // ---- rho and Theta
+#pragma unroll 1
+    for (int x = 0; x < 2; ++x) {
+        const int k = k0 + 4 * x;
+        const int64_t node = node0 + x * NT;
+        int sl[3], ln[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            sl[d] = dir_slot<NQ, double>(d, i, j, k);
+            ln[d] = dir_line<NQ>(d, i, j, k);
+        }
+        double v[2];
+        fixed_sums<NQ>(v, fix.shift, geo.Jinv[node],
+                       [&](int d, int b) { return sF[(d < 2 ? 5 * d + 4 * b : 10 + b) * N3 + sl[d]]; },
+                       [&](int d, int b) { return (int)sE[(d < 2 ? 5 * d + 4 * b : 10 + b) * NL + ln[d]]; });
+        rhs[node] = v[0];
+        rhs[4 * M + node] = v[1];
     }
 }
 
@@ -156,7 +279,19 @@ cudaError_t launch_kernel(ElemRange r, int nf, const DeviceGeometry &geo, const 
 template <int NQ>
 cudaError_t launch_nq(ElemRange r, int nf, const DeviceGeometry &geo, const NativeParams &P,
                       const FixedTables<16, 4> &fix, const double *q, double *rhs, cudaStream_t s) {
-    if (nf == kFields) return launch_kernel<NQ, false>(r, nf, geo, P, fix, q, rhs, s);
+    if (nf == kFields) {
+        if constexpr (NQ == kEight) {
+            const cudaError_t e = cudaFuncSetAttribute(vol_rhs_fp64_eight_kernel,
+                                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       (int)kEightSmem);
+            if (e != cudaSuccess) return e;
+            vol_rhs_fp64_eight_kernel<<<(unsigned)r.count, kEightThreads, kEightSmem, s>>>(
+                geo, P, fix, q, rhs, r.M, r.e0);
+            return cudaGetLastError();
+        } else {
+            return launch_kernel<NQ, false>(r, nf, geo, P, fix, q, rhs, s);
+        }
+    }
     return launch_kernel<NQ, true>(r, nf, geo, P, fix, q, rhs, s);
 }
 

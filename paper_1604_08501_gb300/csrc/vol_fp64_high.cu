@@ -286,7 +286,7 @@ vol_rhs_high_kernel(typename HighTypes<T>::Geo geo,
                 } else {
                     pp = pressure_perturbation(q[4 * M + node], geo.theta_ref[node], geo.w[node],
                                                geo.A[node], P);
-                    rinv = __drcp_rn(q[node]);
+                    rinv = rcp_fp64(q[node]);
                     Th = q[4 * M + node];
                     sP[k * NL + c] = pp;
                 }
@@ -458,15 +458,21 @@ vol_rhs_high_kernel(typename HighTypes<T>::Geo geo,
                     if (gl >= gn) break;
                     const int b = b0 + gl;
                     const T *F = sF + gl * 3 * FB;
-                    T R;
+                    T v;
                     if constexpr (MIXED) {
-                        R = F[s0] + F[FB + s1] + F[2 * FB + s2];
+                        v = -jinv * (F[s0] + F[FB + s1] + F[2 * FB + s2]);
                     } else {
                         const short *E = sE + gl * 3 * NL;
-                        R = fixed_sum3<NQ>(F[s0], E[NQ * k + j], F[FB + s1], E[NL + NQ * k + i],
-                                           F[2 * FB + s2], E[2 * NL + NQ * j + i], P.fix.shift);
+                        T w[1];
+                        fixed_sums<NQ>(
+                            w, P.fix.shift, jinv,
+                            [&](int d, int) { return F[d == 0 ? s0 : d == 1 ? FB + s1 : 2 * FB + s2]; },
+                            [&](int d, int) {
+                                return (int)E[d == 0 ? NQ * k + j : d == 1 ? NL + NQ * k + i
+                                                                           : 2 * NL + NQ * j + i];
+                            });
+                        v = w[0];
                     }
-                    T v = -jinv * R;
                     if (b == 3) {
                         if constexpr (MIXED)
                             v = fma(-rv[kk], P.grav, v);

@@ -49,8 +49,10 @@ void run(const double *in, double *fixed, double *fp64, double *ref, int *exps) 
     for (int line = 0; line < NL; ++line)
         for (int n = 0; n < NQ; ++n) {
             const int s = slot<NQ, double>(line, n), o = line * NQ + n;
-            fixed[o] = fixed_sum3<NQ>(a[s], exps[line], a[W + s], exps[NL + line], a[2 * W + s],
-                                  exps[2 * NL + line], t.fix.shift);
+            double v[1];
+            fixed_sums<NQ>(v, t.fix.shift, -1.0, [&](int d, int) { return a[d * W + s]; },
+                           [&](int d, int) { return exps[d * NL + line]; });
+            fixed[o] = v[0];
             fp64[o] = b[s] + b[W + s] + b[2 * W + s];
             long double x = 0;
             for (int d = 0; d < 3; ++d)
@@ -80,5 +82,15 @@ extern "C" void sweep_case(int nq, const double *in, double *fixed, double *fp64
         case 14: return run<14>(in, fixed, fp64, ref, exps);
         case 15: return run<15>(in, fixed, fp64, ref, exps);
         case 16: return run<16>(in, fixed, fp64, ref, exps);
+    }
+}
+
+// n values of -y R 2^(e - 1024 - shift) by the integer multiply.
+extern "C" void scale_case(int n, const long long *R, int e, int shift, const double *y, double *out) {
+    for (int k = 0; k < n; ++k) {   // one line's sum, the other directions zero
+        double v[1];
+        const double z = fix_double(R[k]);
+        fixed_sums<8>(v, shift, y[k], [&](int d, int) { return d ? 0.0 : z; }, [&](int, int) { return e; });
+        out[k] = v[0];
     }
 }

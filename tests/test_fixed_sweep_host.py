@@ -109,3 +109,32 @@ def test_largest_sums(lib, nq):
         x[:, line] = np.where(D[line % nq] < 0, -big, big) * (-1) ** (line // nq)
     fix, fp, ref, _ = sweep(lib, nq, x)
     assert np.all(np.abs(fix - ref) <= line_scale(nq, x) * 2.0 ** -55 + 2 * EPS * np.abs(ref))
+
+
+@pytest.mark.parametrize("e", [200, 1023, 1900])
+def test_scaled_sums_round_once(lib, e):
+    """fix_scale against exact rational arithmetic: half a unit in the last place (and the
+    truncation of the product at 2^-63) wherever the result is normal."""
+    from fractions import Fraction
+    rng = np.random.default_rng(e)
+    n, shift = 400, 53
+    R = rng.integers(-3 * 2 ** 60, 3 * 2 ** 60, n) >> rng.integers(0, 62, n)
+    R[:6] = [0, 1, -1, 3 * 2 ** 60, -3 * 2 ** 60, 2 ** 53 + 1]
+    y = rng.standard_normal(n) * 2.0 ** rng.integers(-60, 60, n)
+    y[6:10] = [1.0, -1.0, 2.0, np.nextafter(1.0, 0.0)]
+    if e == 1023:   # factors outside the integer multiply's range
+        y[10:16] = [0.0, 1e-290, 1e290, np.inf, np.nan, -5e-324]
+    out = np.zeros(n)
+    lib.scale_case(n, R.ctypes.data_as(C.c_void_p), e, shift, y.ctypes.data_as(C.c_void_p),
+                   out.ctypes.data_as(C.c_void_p))
+    for k in range(n):
+        if not np.isfinite(y[k]) or y[k] == 0.0 or R[k] == 0:
+            if R[k] != 0:
+                assert np.isnan(out[k]) == np.isnan(y[k]) and np.isinf(out[k]) == np.isinf(y[k])
+            continue
+        want = -Fraction(float(y[k])) * int(R[k]) * Fraction(2) ** (e - 1024 - shift)
+        if not Fraction(2) ** -1021 < abs(want) < Fraction(2) ** 1022:
+            continue
+        got = Fraction(float(out[k]))
+        ulp = Fraction(2) ** (int(np.frexp(out[k])[1]) - 53)
+        assert abs(got - want) <= ulp * (Fraction(1, 2) + Fraction(1, 2 ** 9)), (k, R[k], y[k])
