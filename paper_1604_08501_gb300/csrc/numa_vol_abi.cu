@@ -518,13 +518,16 @@ int numa_vol_rhs_host(numa_vol *h, const void *q, void *rhs) {
     const char *hq = static_cast<const char *>(q);
     char *hr = static_cast<char *>(rhs);
     const int64_t n3 = (int64_t)h->Nq * h->Nq * h->Nq;
-    // Native FP64: 64 chunks (the kernel dominates; a shorter fill and drain).
-    // Double-float and FP32 states: 16 (the copies dominate; fewer, larger
-    // copies).  Measured on GB300 (pinned host memory, 193-210 GB/s each way,
-    // 341 GB/s both at once): double-float 3.84 GDOF/s end to end against
-    // 3.15-3.64 with 64 chunks, mixed 7.38 against 7.08 with 32.
+    // Chunks of about 10 MB each way, 4 to 64 of them: each chunk costs its
+    // copies' and its launch's latency, and the first copy in and the last copy
+    // out overlap nothing.  Measured on GB300 (pinned host memory), FP64 and FP32
+    // states at N = 7, us, with 64 / 32 / 16 / 8 / 4 chunks: 10.5 MB 655 / 357 / 213 /
+    // 163 / 153; 84 MB 900 / 785 / 720 / 658 / 716; 283 MB 2313 / 1945 / 1967 /
+    // 2014 / 2190; FP32 5.2 MB 429 / 237 / 152 / 118 / 101; 42 MB 543 / 465 / 402 /
+    // 388 / 379; 142 MB 1170 / 1186 / 1080 / 1039 / 1078.  The kernels no longer
+    // bound the path, as they did for FP64 when it took 64 chunks.
     const int64_t target =
-        h->elem == sizeof(double) && h->kernel != numa::Kernel::DoubleFloat ? numa_vol::kChunks : 16;
+        std::min<int64_t>(numa_vol::kChunks, std::max<int64_t>(4, (int64_t)(bytes / (10 << 20))));
     const int chunks = (int)std::min<int64_t>(target, h->Ne);
     const size_t plane = h->elem * h->M;
     // One 2D copy per chunk and direction moves the chunk's slice of every
