@@ -171,10 +171,22 @@ __host__ __device__ __attribute__((noinline)) void sweep_line_fp64_call(double *
 struct FixedSum {
     long long h, m;
 };
+// x y + z, 32 x 32 + 64 bits.  In C the compiler loses sight of the operands' 32
+// bits (an E cut by a mask is a 64-bit value to it) and multiplies 64 by 64:
+// 256 multiplies a line at Nq = 8 instead of 96.
+__host__ __device__ __forceinline__ long long fix_mad_wide(int x, int y, long long z) {
+#ifdef __CUDA_ARCH__
+    long long r;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(x), "r"(y), "l"(z));
+    return r;
+#else
+    return (long long)x * y + z;
+#endif
+}
 __host__ __device__ __forceinline__ void fix_mad(FixedSum &a, int Eh, int El, int Dh, int Dl) {
-    a.h += (long long)Eh * Dh;
-    a.m += (long long)Eh * Dl;
-    a.m += (long long)El * Dh;
+    a.h = fix_mad_wide(Eh, Dh, a.h);
+    a.m = fix_mad_wide(Eh, Dl, a.m);
+    a.m = fix_mad_wide(El, Dh, a.m);
 }
 __host__ __device__ __forceinline__ long long fix_value(FixedSum a) {
     return a.h + (a.m >> kFixLow);
