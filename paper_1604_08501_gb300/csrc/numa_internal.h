@@ -21,12 +21,16 @@ cudaError_t launch_reference_eos(const double *theta_ref, double *w, double *A, 
 cudaError_t launch_vol_rhs_fp64_high(int N, int nf, ElemRange r, const DeviceGeometry &geo,
                                      const HighParams &P, const double *q, double *rhs,
                                      cudaStream_t s);
-// Mixed precision for N = 8..15 (vol_fp64_high.cu, FP32 instantiation: a
-// five-field and an eight-field form, chosen by nf; num_sms sets the
-// distance of its L2 prefetch, one wave of resident CTAs).
+// Mixed precision for N = 8..15 (vol_mixed_high.cu: a thread walks the k-planes
+// of its column; num_sms sets the distance of its L2 prefetch, one wave of
+// resident CTAs), and the whole-element kernel it leaves small meshes and some
+// forms to (vol_fp64_high.cu, FP32 instantiation).
 cudaError_t launch_vol_rhs_mixed_high(int N, int nf, ElemRange r, const MixedGeometry &geo,
                                       const HighParams32 &P, const float *q, float *rhs,
                                       int num_sms, cudaStream_t s);
+cudaError_t launch_vol_rhs_mixed_element(int N, int nf, ElemRange r, const MixedGeometry &geo,
+                                         const HighParams32 &P, const float *q, float *rhs,
+                                         int num_sms, cudaStream_t s);
 cudaError_t launch_vol_rhs_fp64(int N, int nf, ElemRange r, const DeviceGeometry &geo,
                                 const NativeParams &P, const FixedTables<16, 4> &fix,
                                 const double *q, double *rhs, cudaStream_t s);

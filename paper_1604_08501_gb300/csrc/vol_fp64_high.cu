@@ -29,6 +29,9 @@
 // fields, N = 11 1.405 -> 0.685 ms, N = 15 1.569 -> 0.839 ms, with three tracers
 // 2.100 -> 0.951 and 2.365 -> 1.200 ms; what is left is bound by the latency of
 // the passes' loads and barriers (a field at a time), no longer by the FP64 pipe.
+// (Meshes of two elements per SM and more run the mixed mode in
+// vol_mixed_high.cu where that is faster; a few elements finish sooner here, with
+// three or four threads per column.)
 // Shared memory at Nq = 16: 226 KB in FP64, 204 KB in the mixed mode (FP32 perturbation
 // state and arithmetic as vol_mixed.cu).
 #include <cuda_runtime.h>
@@ -556,9 +559,10 @@ cudaError_t launch_vol_rhs_fp64_high(int N, int nf, ElemRange r, const DeviceGeo
     return launch_high_order<double>(N, nf, r, geo, P, q, rhs, 0, s);
 }
 
-cudaError_t launch_vol_rhs_mixed_high(int N, int nf, ElemRange r, const MixedGeometry &geo,
-                                      const HighParams32 &P, const float *q, float *rhs,
-                                      int num_sms, cudaStream_t s) {
+// The meshes and forms that vol_mixed_high.cu leaves to this kernel.
+cudaError_t launch_vol_rhs_mixed_element(int N, int nf, ElemRange r, const MixedGeometry &geo,
+                                         const HighParams32 &P, const float *q, float *rhs,
+                                         int num_sms, cudaStream_t s) {
     return launch_high_order<float>(N, nf, r, geo, P, q, rhs, num_sms, s);
 }
 
