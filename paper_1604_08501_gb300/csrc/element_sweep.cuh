@@ -65,16 +65,19 @@ template <int NQ>
 __host__ __device__ constexpr int element_threads() {
     return NQ == 2 ? 8 : (NQ * NQ * NQ + 31) / 32 * 32;
 }
-// Elements per CTA: CTAs of 256 threads at Nq = 2, 3 and 4, one element from
+// Elements per CTA: CTAs of 128 threads at Nq = 2, 3 and 4, one element from
 // Nq = 5.  An SM holds 32 CTAs, a quarter of its threads where a CTA is one
-// Nq = 2 element: 96^3 of them, one and 32 a CTA, take 449 and 99 us in
-// NUMA_MIXED, 6.10 and 1.50 ms in NUMA_FP64; 64^3 at Nq = 3 141 and 121 us (one
-// and 8 a CTA, the L2 prefetch with them); Nq = 4 is the same either way.  Two and
-// four elements a CTA at Nq = 5 and 6 were slower (N = 4, 54.7 to 65 us against
-// 53.4; N = 5 61.6 against 54.2): the CTA's barriers wait for more warps.
+// Nq = 2 element: 96^3 of them, one and 16 a CTA, take 449 and 97 us in
+// NUMA_MIXED, 6.10 and 1.43 ms in NUMA_FP64; 64^3 at Nq = 3 141 and 123 us (one
+// and 4 a CTA, the L2 prefetch with them), 48x48x24 at Nq = 4 50.2 and 49.6 us,
+// FP64 325 us with four and 319 with two.  Twice as many elements a CTA leave SMs
+// idle on small meshes (512 elements of Nq = 2 in NUMA_FP64 12.3 us with 32,
+// 8.4 with 16); two and four a CTA at Nq = 5 and 6 were slower (N = 4, 54.7 to
+// 65 us against 53.4; N = 5 61.6 against 54.2): the CTA's barriers wait for more
+// warps.
 template <int NQ>
 __host__ __device__ constexpr int cta_elements() {
-    return NQ == 2 ? 32 : NQ == 3 ? 8 : NQ == 4 ? 4 : 1;
+    return NQ == 2 ? 16 : NQ == 3 ? 4 : NQ == 4 ? 2 : 1;
 }
 template <int NQ>
 __host__ __device__ constexpr int cta_threads() {   // one element: a thread per point, no padding

@@ -58,13 +58,16 @@ struct DfShape {
     static constexpr int kItems = kFields * 3 * NL;    // (direction, field, line) sweep tasks
 };
 
-// Resident CTAs per SM the register budget is sized for: two 512-thread CTAs
-// at Nq = 8 (64 registers); about 640 threads per SM at the other orders
-// (about 100 registers: the double-float sweeps of one line need more than
-// 64 without spilling), at most 32 CTAs.
+// Resident CTAs per SM the register budget is sized for: about 1024 threads at
+// every order (56 to 72 registers, up to 100 bytes spilled), at most 32 CTAs.
+// The spills cost less than the warps they buy: 3.5 million points, us, at 640,
+// 704, 864 and 1029 threads per SM (Nq = 7: one, two, two and three CTAs):
+// Nq = 3 471 432 412 412, 4 198 185 178 178, 5 251 250 229 199, 6 321 235 207
+// 207, 7 461 304 304 261; three tracers 7 743 448 448 386, 5 399 399 360 320.
+// (With 1280 and 1536 threads Nq = 4, 6 and the tracer forms get slower.)
 template <int NQ>
 constexpr int df_min_ctas() {
-    constexpr int n = NQ == 8 ? 2 : 640 / (NQ * NQ * NQ);
+    constexpr int n = 1029 / (NQ * NQ * NQ);
     return n < 1 ? 1 : (n > 32 ? 32 : n);
 }
 
