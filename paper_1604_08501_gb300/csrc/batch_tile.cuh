@@ -24,7 +24,7 @@ constexpr int kThreads = 512;
 // run beside the other's FP64 phases (the FP64 pipe binds, about 72 operations
 // per point and stage).  Measured on 6 instances, 4.6 million points, ten steps
 // (50 stages): 75.5 ms with FP64 sweeps, q and dq in registers and one CTA per SM,
-// 36.5 ms so.  The tracer form keeps the base fields' q and dq in registers
+// 29.7 ms so.  The tracer form keeps the base fields' q and dq in registers
 // (98 KB of fluxes: one CTA per SM).  Mixed: the fluxes, q and dq (10 values) and the point's geometry
 // (g and Jinv, 10 values) in shared memory, so that the kernel fits 64
 // registers and two CTAs share an SM, twice the warps to hide latency.
@@ -329,16 +329,25 @@ __device__ void run_tile(const BatchInstance &I, int64_t e0, int64_t count,
                         jinv = jinv_g;
                         drho = Q(0) - rho_ref_g;
                     }
-                    T v[kFields];
-                    sums(v, 0, jinv);
+                    // dq and q of fields b0 .. from dt times their rhs
+                    auto update = [&](auto &v, int b0) {
+                        constexpr int NB = sizeof(v) / sizeof(T);
+                        sums(v, b0, jinv);
 #pragma unroll
-                    for (int b = 0; b < kFields; ++b) {
-                        T rhs = v[b];
-                        if (b == 3) rhs = fma(-drho, grav, rhs);
-                        const T d = fma(a, DQ(b), dtt * rhs);
-                        DQ(b) = d;
-                        Q(b) = fma(bcoef, d, Q(b));
-                    }
+                        for (int b = b0; b < b0 + NB; ++b) {
+                            T rhs = v[b - b0];
+                            if (b == 3) rhs = fma(-drho, grav, rhs);
+                            const T d = fma(a, DQ(b), dtt * rhs);
+                            DQ(b) = d;
+                            Q(b) = fma(bcoef, d, Q(b));
+                        }
+                    };
+                    // in two groups: the integer chains of all five fields side by
+                    // side spill at 64 registers (FP64: 32.9 ms in one group,
+                    // 29.7 in two, 30.1 in three, on the 6 instances above)
+                    T v3[3], v2[2];
+                    update(v3, 0);
+                    update(v2, 3);
                     if constexpr (TR) {
 #pragma unroll
                         for (int t = 0; t < NTR; ++t) {

@@ -34,7 +34,9 @@
 //    million points N = 3 383 -> 325 us, N = 4 397 -> 332 us, N = 5 394 -> 334 us;
 //    N = 7 needed smaller CTAs as well (vol_rhs_fp64_eight_kernel): 32768
 //    elements 1.881 -> 1.656 ms, the FP64 pipe 76 % busy of the 83 % that a loop of
-//    DFMAs reaches.
+//    DFMAs reaches.  Later steps (fix_mad_wide; these sums in two groups of
+//    fields): N = 7 1.533 ms, N = 3 318 us, N = 4 330 us, 512 elements of N = 4
+//    12.3 us a call.
 //
 // One CTA of Nq^3 threads per element (several elements from Nq = 6 down, so
 // that a CTA has a few hundred threads: cta_elements), in three phases: fluxes by point,
@@ -150,12 +152,20 @@ vol_rhs_fp64_kernel(DeviceGeometry geo, const __grid_constant__ NativeParams P,
         sl[d] = d * nf * EW + el * N3 + dir_slot<NQ, double>(d, i, j, k);
         ln[d] = d * nf * EL + el * NL + dir_line<NQ>(d, i, j, k);
     }
-    double v[kFields];
-    fixed_sums<NQ>(v, fix.shift, Jinv, [&](int d, int b) { return sF[sl[d] + b * EW]; },
-                   [&](int d, int b) { return (int)sE[ln[d] + b * EL]; });
-    v[3] = fma(-drho, P.eos.grav, v[3]);
+    auto store = [&](auto &v, int b0) {   // fields b0 ..
+        constexpr int NB = sizeof(v) / sizeof(double);
+        fixed_sums<NQ>(v, fix.shift, Jinv, [&](int d, int b) { return sF[sl[d] + (b0 + b) * EW]; },
+                       [&](int d, int b) { return (int)sE[ln[d] + (b0 + b) * EL]; });
 #pragma unroll
-    for (int b = 0; b < kFields; ++b) rhs[b * M + node] = v[b];
+        for (int b = 0; b < NB; ++b) {
+            if (b0 + b == 3) v[b] = fma(-drho, P.eos.grav, v[b]);
+            rhs[(b0 + b) * M + node] = v[b];
+        }
+    };
+    // two groups: five fields' integer chains side by side spill at 64 registers
+    double v3[3], v2[2];
+    store(v3, 0);
+    store(v2, 3);
     if constexpr (TRACERS) {
 #pragma unroll
         for (int b = kFields; b < kMaxFields; ++b) {
