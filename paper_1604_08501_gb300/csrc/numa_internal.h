@@ -33,7 +33,7 @@ cudaError_t launch_vol_rhs_mixed_element(int N, int nf, ElemRange r, const Mixed
                                          int num_sms, cudaStream_t s);
 cudaError_t launch_vol_rhs_fp64(int N, int nf, ElemRange r, const DeviceGeometry &geo,
                                 const NativeParams &P, const FixedTables<16, 4> &fix,
-                                const double *q, double *rhs, cudaStream_t s);
+                                const double *q, double *rhs, int num_sms, cudaStream_t s);
 
 // Launchers of the double-float path (vol_df64.cu).  abs_max: max |src| into
 // *amax_bits (the bit pattern of a nonnegative double).  to_df: split src

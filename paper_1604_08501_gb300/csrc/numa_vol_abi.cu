@@ -461,7 +461,8 @@ cudaError_t launch(numa_vol *h, const void *q, void *rhs, int64_t e0, int64_t co
                                               static_cast<const double *>(q),
                                               static_cast<double *>(rhs), s);
     return numa::launch_vol_rhs_fp64(h->N, h->nf, r, h->geo, h->nparams,
-                                     h->nfix, static_cast<const double *>(q), static_cast<double *>(rhs), s);
+                                     h->nfix, static_cast<const double *>(q), static_cast<double *>(rhs),
+                                     h->num_sms, s);
 }
 
 }  // namespace

@@ -135,54 +135,63 @@ __device__ __noinline__ double eos_pressure_fp64(double Th, const DfParams &P) {
     return __dmul_rn(P.p0, pow(__ddiv_rn(__dmul_rn(P.R, Th), P.p0), P.gamma));
 }
 
-// Native FP64 evaluation of one element from df-stored geometry (rare path).
-template <int NQ, bool TR>
+// Native FP64 evaluation of one element from df-stored geometry (rare path), a
+// field at a time in 3 Nq^3 values of shared memory; NT threads, each with the
+// points threadIdx.x, threadIdx.x + NT, ...
+template <int NQ, int NT>
 __device__ void element_fp64(const DfGeometry &geo, const DfParams &P, const double *__restrict__ q,
-                             double *__restrict__ rhs, int64_t M, int64_t e, int nf, double *sF) {
+                             double *rhs, int64_t M, int64_t e, int nf, double *sF) {
     constexpr int N3 = DfShape<NQ>::N3;
-    const int NF = TR ? nf : kFields;   // flux blocks per direction
-    const int l = threadIdx.x;
-    const int64_t node = e * N3 + l;
-    __syncthreads();  // sF aliases the df buffers of the caller
-    const double rho = q[node];
-    const double U1 = q[M + node], U2 = q[2 * M + node], U3 = q[3 * M + node];
-    const double Th = q[4 * M + node];
-    const double pp = eos_pressure_fp64(Th, P) - eos_pressure_fp64(geo.theta_ref[node], P);
+    constexpr int PPT = (N3 + NT - 1) / NT;
+    double u[PPT][3], pp[PPT];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const double g1 = df_to_double(ld_df(geo.g[3 * d], node));
-        const double g2 = df_to_double(ld_df(geo.g[3 * d + 1], node));
-        const double g3 = df_to_double(ld_df(geo.g[3 * d + 2], node));
-        const double u = (g1 * U1 + g2 * U2 + g3 * U3) / rho;
-        double *F = sF + d * NF * N3 + l;
-        F[0 * N3] = rho * u;
-        F[1 * N3] = U1 * u + g1 * pp;
-        F[2 * N3] = U2 * u + g2 * pp;
-        F[3 * N3] = U3 * u + g3 * pp;
-        F[4 * N3] = Th * u;
-        if constexpr (TR) {
-            for (int b = kFields; b < nf; ++b) F[b * N3] = q[b * M + node] * u;   // tracers Q u_d
+    for (int x = 0; x < PPT; ++x) {
+        const int l = threadIdx.x + x * NT;
+        const int64_t node = e * N3 + l;
+        pp[x] = eos_pressure_fp64(q[4 * M + node], P) - eos_pressure_fp64(geo.theta_ref[node], P);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const double g1 = df_to_double(ld_df(geo.g[3 * d], node));
+            const double g2 = df_to_double(ld_df(geo.g[3 * d + 1], node));
+            const double g3 = df_to_double(ld_df(geo.g[3 * d + 2], node));
+            u[x][d] = (g1 * q[M + node] + g2 * q[2 * M + node] + g3 * q[3 * M + node]) / q[node];
         }
     }
-    __syncthreads();
-    const int i = l % NQ, j = (l / NQ) % NQ, k = l / (NQ * NQ);
-    const double Jinv = df_to_double(ld_df(geo.Jinv, node));
-    const double drho = rho - geo.rho_ref[node];
 #pragma unroll 1
-    for (int b = 0; b < NF; ++b) {
-        const double *Fr = sF + (0 * NF + b) * N3;
-        const double *Fs = sF + (1 * NF + b) * N3;
-        const double *Ft = sF + (2 * NF + b) * N3;
-        double s = 0.0;
+    for (int b = 0; b < nf; ++b) {
+        __syncthreads();  // sF aliases the df buffers of the caller, then the last field's fluxes
 #pragma unroll
-        for (int n = 0; n < NQ; ++n) s += P.D[i * NQ + n] * Fr[(k * NQ + j) * NQ + n];
+        for (int x = 0; x < PPT; ++x) {
+            const int l = threadIdx.x + x * NT;
+            const int64_t node = e * N3 + l;
+            const double qb = q[b * M + node];
 #pragma unroll
-        for (int n = 0; n < NQ; ++n) s += P.D[j * NQ + n] * Fs[(k * NQ + n) * NQ + i];
+            for (int d = 0; d < 3; ++d) {
+                double F = qb * u[x][d];
+                if (b >= 1 && b <= 3) {
+                    const float2 *g = b == 1 ? geo.g[3 * d] : b == 2 ? geo.g[3 * d + 1] : geo.g[3 * d + 2];
+                    F += df_to_double(ld_df(g, node)) * pp[x];
+                }
+                sF[d * N3 + l] = F;
+            }
+        }
+        __syncthreads();
 #pragma unroll
-        for (int n = 0; n < NQ; ++n) s += P.D[k * NQ + n] * Ft[(n * NQ + j) * NQ + i];
-        double v = -Jinv * s;
-        if (b == 3) v -= drho * P.grav;
-        rhs[b * M + node] = v;
+        for (int x = 0; x < PPT; ++x) {
+            const int l = threadIdx.x + x * NT;
+            const int64_t node = e * N3 + l;
+            const int i = l % NQ, j = (l / NQ) % NQ, k = l / (NQ * NQ);
+            double s = 0.0;
+#pragma unroll
+            for (int n = 0; n < NQ; ++n) s += P.D[i * NQ + n] * sF[(k * NQ + j) * NQ + n];
+#pragma unroll
+            for (int n = 0; n < NQ; ++n) s += P.D[j * NQ + n] * sF[N3 + (k * NQ + n) * NQ + i];
+#pragma unroll
+            for (int n = 0; n < NQ; ++n) s += P.D[k * NQ + n] * sF[2 * N3 + (n * NQ + j) * NQ + i];
+            double v = -df_to_double(ld_df(geo.Jinv, node)) * s;
+            if (b == 3) v -= (q[node] - geo.rho_ref[node]) * P.grav;
+            rhs[b * M + node] = v;
+        }
     }
 }
 
@@ -207,65 +216,27 @@ __device__ __forceinline__ void prefetch_element(const DfGeometry &geo, const do
     }
 }
 
-// ahead: half the CTAs resident on the GPU at once.  The element that many
-// launch slots later starts soon on some SM, so its arrays are prefetched to
-// L2 now and its loads then hit L2 rather than DRAM (one wave ahead: 1.30 ->
-// 1.22 ms at N = 7, 32768 elements; half a wave 14.06 against 13.91 GDOF/s
-// for one wave and 13.98 for a quarter; two waves ahead was slower than
-// none, the prefetched data displacing the running wave's).
-// TR: the 8-field form (nf = 5 + tracers, 6..8): the tracers' state is split
-// like the other fields and their fluxes are Q u_d; nf blocks per direction.
-template <int NQ, bool TR>
-__global__ void __launch_bounds__(NQ * NQ * NQ, df_min_ctas<NQ>())
-vol_rhs_df64_kernel(DfGeometry geo, DfParams P, const double *__restrict__ q,
-                    double *__restrict__ rhs, int64_t M, int64_t e0, int64_t e_end,
-                    int64_t ahead, int nf) {
-    constexpr int N3 = DfShape<NQ>::N3;
-    constexpr int NL = DfShape<NQ>::NL;
-    constexpr int HALF = NQ / 2;
-    constexpr bool ODD = (NQ & 1) != 0;
-    constexpr int C = NQ / 2;
-    constexpr int NT = kMaxFields - kFields;   // tracers at most
-    const int NF = TR ? nf : kFields;          // flux blocks per direction
-    extern __shared__ float2 sbuf[];  // [direction*NF + field][slot], 3 NF Nq^3 float2
-    const int l = threadIdx.x;
-    const int i = l % NQ, j = (l / NQ) % NQ, k = l / (NQ * NQ);
-    const int64_t e = e0 + blockIdx.x;
-    const int64_t node = e * N3 + l;
-    if (l == 0 && e + ahead < e_end) prefetch_element<NQ>(geo, q, M, NF, e + ahead);
-
-    // ---- phase 1: state, p', fluxes -----------------------------------
-    bool big = false, tiny = false;
+// Fluxes of one point (the first five fields): put(d, b, F).  big is set where the
+// state leaves the split range or rho is not positive; u3 gets the contravariant
+// velocities, drho rho - rho_ref.
+template <typename Put>
+__device__ __forceinline__ void df_point_fluxes(const DfGeometry &geo, const DfParams &P,
+                                                const double *__restrict__ q, int64_t M, int64_t node,
+                                                bool &big, df (&u3)[3], df &drho, Put put) {
+    bool tiny = false;
     df Q[kFields];
     double qd[kFields];
 #pragma unroll
     for (int b = 0; b < kFields; ++b) qd[b] = q[b * M + node];
 #pragma unroll
     for (int b = 0; b < kFields; ++b) Q[b] = df_split(qd[b], big, tiny);
-    df QT[TR ? NT : 1];   // the tracers
-    if constexpr (TR) {
-#pragma unroll
-        for (int t = 0; t < NT; ++t)
-            QT[t] = kFields + t < nf ? df_split(q[(kFields + t) * M + node], big, tiny)
-                                     : df{0.0f, 0.0f};
-    }
     // Exact FP64 differences (Sterbenz: the operands are within a factor 2 in
     // the fast path) before splitting, so the perturbations keep full accuracy.
     const double th0 = geo.theta_ref[node];
-    const double thp_d = qd[4] - th0;
-    const double drho_d = qd[0] - geo.rho_ref[node];
-    const df thp = df_split(thp_d, big, tiny);
-    const df drho = df_split(drho_d, big, tiny);
-    const bool bad = big || !(qd[0] > 0.0);
-    if (__syncthreads_or(bad)) {
-        element_fp64<NQ, TR>(geo, P, q, rhs, M, e, nf, reinterpret_cast<double *>(sbuf));
-        return;
-    }
-
+    const df thp = df_split(qd[4] - th0, big, tiny);
+    drho = df_split(qd[0] - geo.rho_ref[node], big, tiny);
+    big = big || !(qd[0] > 0.0);
     const df rinv = df_rcp(Q[0]);
-    // J^-1 here rather than after the sweeps: its load overlaps phase 1
-    // (13.90 against 13.74 GDOF/s at N = 7)
-    const df jinv = ld_df(geo.Jinv, node);
     df pp;
     {
         const df x = df_mul(thp, ld_df(geo.w, node));
@@ -276,7 +247,6 @@ vol_rhs_df64_kernel(DfGeometry geo, DfParams P, const double *__restrict__ q,
             pp = df_split(eos_pressure_fp64(qd[4], P) - eos_pressure_fp64(th0, P), b2, t2);
         }
     }
-
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         const df g1 = ld_df(geo.g[3 * d], node);
@@ -287,89 +257,140 @@ vol_rhs_df64_kernel(DfGeometry geo, DfParams P, const double *__restrict__ q,
         dot2_add(acc, g3, Q[3]);
         const df v = dot2_value(acc);
         const df u = df_mul(df_norm(v), rinv);
-        df F[kFields];
-        F[0] = v;
-        {
-            dot2 a = dot2_first(Q[1], u);
-            dot2_add(a, g1, pp);
-            F[1] = dot2_value(a);
-            dot2 b = dot2_first(Q[2], u);
-            dot2_add(b, g2, pp);
-            F[2] = dot2_value(b);
-            dot2 c = dot2_first(Q[3], u);
-            dot2_add(c, g3, pp);
-            F[3] = dot2_value(c);
+        u3[d] = u;
+        put(d, 0, v);
+        dot2 a = dot2_first(Q[1], u);
+        dot2_add(a, g1, pp);
+        put(d, 1, dot2_value(a));
+        dot2 b = dot2_first(Q[2], u);
+        dot2_add(b, g2, pp);
+        put(d, 2, dot2_value(b));
+        dot2 c = dot2_first(Q[3], u);
+        dot2_add(c, g3, pp);
+        put(d, 3, dot2_value(c));
+        put(d, 4, df_mul(Q[4], u));
+    }
+}
+
+// Even-odd D sweep of one line, in place.
+template <int NQ>
+__device__ __forceinline__ void df_sweep_line(float2 *buf, int line, const DfParams &P) {
+    constexpr int HALF = NQ / 2;
+    constexpr bool ODD = (NQ & 1) != 0;
+    constexpr int C = NQ / 2;
+    df F[NQ];
+#pragma unroll
+    for (int n = 0; n < NQ; ++n) {
+        const float2 v = buf[slot<NQ>(line, n)];
+        F[n] = df{v.x, v.y};
+    }
+    df E[HALF], O[HALF];
+#pragma unroll
+    for (int m = 0; m < HALF; ++m) {
+        E[m] = df_add(F[m], F[NQ - 1 - m]);
+        O[m] = df_sub(F[m], F[NQ - 1 - m]);
+    }
+#pragma unroll
+    for (int r = 0; r < HALF; ++r) {
+        dot2 a = dot2_first(P.De[r][0], E[0]);
+        dot2 b = dot2_first(P.Do[r][0], O[0]);
+#pragma unroll
+        for (int m = 1; m < HALF; ++m) {
+            dot2_add(a, P.De[r][m], E[m]);
+            dot2_add(b, P.Do[r][m], O[m]);
         }
-        F[4] = df_mul(Q[4], u);
-        const int s = dir_slot<NQ>(d, i, j, k);
+        if constexpr (ODD) dot2_add(a, P.Dc[r], F[C]);
+        const df A = dot2_value(a), B = dot2_value(b);
+        const df Si = df_add(B, A);
+        const df Sm = df_sub(B, A);
+        buf[slot<NQ>(line, r)] = make_float2(Si.h, Si.l);
+        buf[slot<NQ>(line, NQ - 1 - r)] = make_float2(Sm.h, Sm.l);
+    }
+    if constexpr (ODD) {
+        dot2 c = dot2_first(P.Dcr[0], O[0]);
 #pragma unroll
-        for (int b = 0; b < kFields; ++b) sbuf[(d * NF + b) * N3 + s] = make_float2(F[b].h, F[b].l);
-        if constexpr (TR) {
+        for (int m = 1; m < HALF; ++m) dot2_add(c, P.Dcr[m], O[m]);
+        const df Sc = df_norm(dot2_value(c));
+        buf[slot<NQ>(line, C)] = make_float2(Sc.h, Sc.l);
+    }
+}
+
+// -J^-1 times the sum of a point's three sweeps, and the gravity source (U3).
+__device__ __forceinline__ double df_combine(float2 r, float2 s, float2 t, df jinv, bool grav,
+                                             df drho, const DfParams &P, bool &finite) {
+    const df R = df_add(df_add(df{r.x, r.y}, df{s.x, s.y}), df{t.x, t.y});
+    df v = df_mul(df_norm(R), jinv);
+    if (grav) v = df_add(v, df_mul(drho, P.grav_df));
+    v = df_norm(v);
+    finite = finite && isfinite(v.h) && isfinite(v.l);
+    return -df_to_double(v);
+}
+
+// ahead: half the CTAs resident on the GPU at once.  The element that many
+// launch slots later starts soon on some SM, so its arrays are prefetched to
+// L2 now and its loads then hit L2 rather than DRAM (one wave ahead: 1.30 ->
+// 1.22 ms at N = 7, 32768 elements; half a wave 14.06 against 13.91 GDOF/s
+// for one wave and 13.98 for a quarter; two waves ahead was slower than
+// none, the prefetched data displacing the running wave's).
+// TR: the 8-field form (nf = 5 + tracers, 6..8): the tracers' state is split
+// like the other fields and their fluxes are Q u_d; nf blocks per direction.
+template <int NQ, bool TR>
+__global__ void __launch_bounds__(NQ * NQ * NQ, df_min_ctas<NQ>())
+vol_rhs_df64_kernel(DfGeometry geo, const __grid_constant__ DfParams P, const double *__restrict__ q,
+                    double *__restrict__ rhs, int64_t M, int64_t e0, int64_t e_end,
+                    int64_t ahead, int nf) {
+    constexpr int N3 = DfShape<NQ>::N3;
+    constexpr int NL = DfShape<NQ>::NL;
+    constexpr int NT = kMaxFields - kFields;   // tracers at most
+    const int NF = TR ? nf : kFields;          // flux blocks per direction
+    extern __shared__ float2 sbuf[];  // [direction*NF + field][slot], 3 NF Nq^3 float2
+    const int l = threadIdx.x;
+    const int i = l % NQ, j = (l / NQ) % NQ, k = l / (NQ * NQ);
+    const int64_t e = e0 + blockIdx.x;
+    const int64_t node = e * N3 + l;
+    if (l == 0 && e + ahead < e_end) prefetch_element<NQ>(geo, q, M, NF, e + ahead);
+
+    // ---- phase 1: state, p', fluxes -----------------------------------
+    bool bad = false;
+    df u3[3], drho;
+    int sl[3];
 #pragma unroll
-            for (int t = 0; t < NT; ++t) {
-                if (kFields + t >= nf) break;
-                const df Ft = df_mul(QT[t], u);
-                sbuf[(d * NF + kFields + t) * N3 + s] = make_float2(Ft.h, Ft.l);
+    for (int d = 0; d < 3; ++d) sl[d] = d * NF * N3 + dir_slot<NQ>(d, i, j, k);
+    // J^-1 here rather than after the sweeps: its load overlaps phase 1
+    // (13.90 against 13.74 GDOF/s at N = 7)
+    const df jinv = ld_df(geo.Jinv, node);
+    df_point_fluxes(geo, P, q, M, node, bad, u3, drho, [&](int d, int b, df F) {
+        sbuf[sl[d] + b * N3] = make_float2(F.h, F.l);
+    });
+    if constexpr (TR) {   // the tracers
+#pragma unroll
+        for (int t = 0; t < NT; ++t) {
+            if (kFields + t >= nf) break;
+            bool tiny = false;
+            const df Qt = df_split(q[(kFields + t) * M + node], bad, tiny);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const df Ft = df_mul(Qt, u3[d]);
+                sbuf[sl[d] + (kFields + t) * N3] = make_float2(Ft.h, Ft.l);
             }
         }
     }
-    __syncthreads();
+    if (__syncthreads_or(bad)) {
+        element_fp64<NQ, N3>(geo, P, q, rhs, M, e, NF, reinterpret_cast<double *>(sbuf));
+        return;
+    }
 
     // ---- phase 2: even-odd D sweeps, one line per task -----------------
-    for (int item = l; item < (TR ? 3 * NF * NL : DfShape<NQ>::kItems); item += N3) {
-        float2 *buf = sbuf + (item / NL) * N3;
-        const int line = item % NL;
-        df F[NQ];
-#pragma unroll
-        for (int n = 0; n < NQ; ++n) {
-            const float2 v = buf[slot<NQ>(line, n)];
-            F[n] = df{v.x, v.y};
-        }
-        df E[HALF], O[HALF];
-#pragma unroll
-        for (int m = 0; m < HALF; ++m) {
-            E[m] = df_add(F[m], F[NQ - 1 - m]);
-            O[m] = df_sub(F[m], F[NQ - 1 - m]);
-        }
-#pragma unroll
-        for (int r = 0; r < HALF; ++r) {
-            dot2 a = dot2_first(P.De[r][0], E[0]);
-            dot2 b = dot2_first(P.Do[r][0], O[0]);
-#pragma unroll
-            for (int m = 1; m < HALF; ++m) {
-                dot2_add(a, P.De[r][m], E[m]);
-                dot2_add(b, P.Do[r][m], O[m]);
-            }
-            if constexpr (ODD) dot2_add(a, P.Dc[r], F[C]);
-            const df A = dot2_value(a), B = dot2_value(b);
-            const df Si = df_add(B, A);
-            const df Sm = df_sub(B, A);
-            buf[slot<NQ>(line, r)] = make_float2(Si.h, Si.l);
-            buf[slot<NQ>(line, NQ - 1 - r)] = make_float2(Sm.h, Sm.l);
-        }
-        if constexpr (ODD) {
-            dot2 c = dot2_first(P.Dcr[0], O[0]);
-#pragma unroll
-            for (int m = 1; m < HALF; ++m) dot2_add(c, P.Dcr[m], O[m]);
-            const df Sc = df_norm(dot2_value(c));
-            buf[slot<NQ>(line, C)] = make_float2(Sc.h, Sc.l);
-        }
-    }
+    for (int item = l; item < (TR ? 3 * NF * NL : DfShape<NQ>::kItems); item += N3)
+        df_sweep_line<NQ>(sbuf + (item / NL) * N3, item % NL, P);
     __syncthreads();
 
     // ---- phase 3: combine, scale, gravity, store -----------------------
     double out[kFields];
     bool finite = true;
     auto field = [&](int b) -> double {
-        const float2 r = sbuf[(0 * NF + b) * N3 + dir_slot<NQ>(0, i, j, k)];
-        const float2 s = sbuf[(1 * NF + b) * N3 + dir_slot<NQ>(1, i, j, k)];
-        const float2 t = sbuf[(2 * NF + b) * N3 + dir_slot<NQ>(2, i, j, k)];
-        df R = df_add(df_add(df{r.x, r.y}, df{s.x, s.y}), df{t.x, t.y});
-        df v = df_mul(df_norm(R), jinv);
-        if (b == 3) v = df_add(v, df_mul(drho, P.grav_df));
-        v = df_norm(v);
-        finite = finite && isfinite(v.h) && isfinite(v.l);
-        return -df_to_double(v);
+        return df_combine(sbuf[sl[0] + b * N3], sbuf[sl[1] + b * N3], sbuf[sl[2] + b * N3], jinv,
+                          b == 3, drho, P, finite);
     };
 #pragma unroll
     for (int b = 0; b < kFields; ++b) out[b] = field(b);
@@ -381,11 +402,100 @@ vol_rhs_df64_kernel(DfGeometry geo, DfParams P, const double *__restrict__ q,
     }
     // An overflow anywhere in the element (float range) sends it to FP64.
     if (__syncthreads_or(!finite)) {
-        element_fp64<NQ, TR>(geo, P, q, rhs, M, e, nf, reinterpret_cast<double *>(sbuf));
+        element_fp64<NQ, N3>(geo, P, q, rhs, M, e, NF, reinterpret_cast<double *>(sbuf));
         return;
     }
 #pragma unroll
     for (int b = 0; b < kFields; ++b) rhs[b * M + node] = out[b];
+}
+
+// N = 7 without tracers: 256 threads per element, two points each, four CTAs per
+// SM instead of two of 512 threads, and 13 of the 15 flux blocks in shared
+// memory, as in vol_rhs_fp64_eight_kernel (vol_fp64.cu): the t fluxes of rho and
+// Theta wait in their outputs' places of rhs until the momenta are done.  The
+// operations are those of vol_rhs_df64_kernel<8>, so the results are the same bit
+// for bit; that kernel takes the launches of fewer than three elements per SM,
+// where a lone element of 512 threads finishes sooner.  Measured, us, 512 threads
+// and these: 125 elements 11.1 13.9, 280 16.4 18.5, 512 28.1 26.8, 1728 71.7 69.8,
+// 6912 254 227, 13824 499 438.
+constexpr int kEightThreads = 256, kEightBlocks = 13;
+constexpr size_t kEightSmem = kEightBlocks * sizeof(float2) * 512;
+__device__ __forceinline__ constexpr int eight_block(int d, int b) { return d < 2 ? 5 * d + b : 9 + b; }
+
+__global__ void __launch_bounds__(kEightThreads, 4)
+vol_rhs_df64_eight_kernel(DfGeometry geo, const __grid_constant__ DfParams P,
+                          const double *__restrict__ q, double *rhs, int64_t M, int64_t e0,
+                          int64_t e_end, int64_t ahead) {
+    constexpr int NQ = 8, N3 = 512, NL = 64, NT = kEightThreads;
+    extern __shared__ float2 sbuf[];   // [block][slot]
+    const int l = threadIdx.x;
+    const int i = l % NQ, j = (l / NQ) % NQ, k0 = l / NL;   // points (i, j, k0) and (i, j, k0 + 4)
+    const int64_t e = e0 + blockIdx.x;
+    const int64_t node0 = e * N3 + l;
+    if (l == 0 && e + ahead < e_end) prefetch_element<NQ>(geo, q, M, kFields, e + ahead);
+
+    bool bad = false, finite = true;
+#pragma unroll 1
+    for (int x = 0; x < 2; ++x) {
+        const int64_t node = node0 + x * NT;
+        int sl[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) sl[d] = dir_slot<NQ>(d, i, j, k0 + 4 * x);
+        df u3[3], drho;
+        df_point_fluxes(geo, P, q, M, node, bad, u3, drho, [&](int d, int b, df F) {
+            const float2 v = make_float2(F.h, F.l);
+            if (d == 2 && (b == 0 || b == 4)) *reinterpret_cast<float2 *>(rhs + b * M + node) = v;
+            else sbuf[eight_block(d, b) * N3 + sl[d]] = v;
+        });
+    }
+    if (__syncthreads_or(bad)) {
+        element_fp64<NQ, NT>(geo, P, q, rhs, M, e, kFields, reinterpret_cast<double *>(sbuf));
+        return;
+    }
+#pragma unroll 1
+    for (int item = l; item < kEightBlocks * NL; item += NT)
+        df_sweep_line<NQ>(sbuf + (item / NL) * N3, item % NL, P);
+    __syncthreads();
+#pragma unroll 1
+    for (int x = 0; x < 2; ++x) {
+        const int64_t node = node0 + x * NT;
+        int sl[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) sl[d] = dir_slot<NQ>(d, i, j, k0 + 4 * x);
+        const float2 f0 = *reinterpret_cast<const float2 *>(rhs + node);
+        const float2 f4 = *reinterpret_cast<const float2 *>(rhs + 4 * M + node);
+        bool big = false, tiny = false;
+        const df drho = df_split(q[node] - geo.rho_ref[node], big, tiny);
+        const df jinv = ld_df(geo.Jinv, node);
+#pragma unroll
+        for (int b = 1; b < 4; ++b)
+            rhs[b * M + node] = df_combine(sbuf[eight_block(0, b) * N3 + sl[0]],
+                                           sbuf[eight_block(1, b) * N3 + sl[1]],
+                                           sbuf[eight_block(2, b) * N3 + sl[2]], jinv, b == 3, drho, P,
+                                           finite);
+        // into blocks 10 and 11, whose slots of this point this thread alone has read
+        sbuf[10 * N3 + sl[2]] = f0;
+        sbuf[11 * N3 + sl[2]] = f4;
+    }
+    __syncthreads();
+    if (l < 2 * NL) df_sweep_line<NQ>(sbuf + (10 + l / NL) * N3, l % NL, P);
+    __syncthreads();
+#pragma unroll 1
+    for (int x = 0; x < 2; ++x) {
+        const int64_t node = node0 + x * NT;
+        int sl[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) sl[d] = dir_slot<NQ>(d, i, j, k0 + 4 * x);
+        const df jinv = ld_df(geo.Jinv, node);
+#pragma unroll
+        for (int b = 0; b < 5; b += 4)
+            rhs[b * M + node] = df_combine(sbuf[b * N3 + sl[0]], sbuf[(5 + b) * N3 + sl[1]],
+                                           sbuf[(10 + b / 4) * N3 + sl[2]], jinv, false, df{0.f, 0.f}, P,
+                                           finite);
+    }
+    // An overflow anywhere in the element (float range) sends it to FP64.
+    if (__syncthreads_or(!finite))
+        element_fp64<NQ, NT>(geo, P, q, rhs, M, e, kFields, reinterpret_cast<double *>(sbuf));
 }
 
 // Largest magnitude of an array (bit patterns of nonnegative doubles order
@@ -457,6 +567,18 @@ template <int NQ>
 cudaError_t launch_df(ElemRange r, int nf, const DfGeometry &geo, const DfParams &P,
                       const double *q, double *rhs, int num_sms, cudaStream_t s) {
     if (nf > kFields) return launch_df_form<NQ, true>(r, nf, geo, P, q, rhs, num_sms, s);
+    if constexpr (NQ == 8) {
+        if (r.count >= 3 * (int64_t)num_sms) {
+            const cudaError_t e = cudaFuncSetAttribute(vol_rhs_df64_eight_kernel,
+                                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       (int)kEightSmem);
+            if (e != cudaSuccess) return e;
+            const int64_t ahead = num_sms > 0 ? 2 * (int64_t)num_sms : 1;   // half a wave
+            vol_rhs_df64_eight_kernel<<<(unsigned)r.count, kEightThreads, kEightSmem, s>>>(
+                geo, P, q, rhs, r.M, r.e0, r.e0 + r.count, ahead);
+            return cudaGetLastError();
+        }
+    }
     return launch_df_form<NQ, false>(r, nf, geo, P, q, rhs, num_sms, s);
 }
 

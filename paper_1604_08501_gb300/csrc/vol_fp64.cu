@@ -186,7 +186,11 @@ vol_rhs_fp64_kernel(DeviceGeometry geo, const __grid_constant__ NativeParams P,
 // in rhs, which nothing else reads or writes meanwhile, until the sums of the
 // momenta are done; they then take two of the momenta's blocks.  Measured, 6912
 // elements: two CTAs of 512 threads 425 us, three of 256 405 us, three of 320
-// 441 us (registers), this 365 us.
+// 441 us (registers), this 365 us.  The operations are those of
+// vol_rhs_fp64_kernel<8>, so the results are the same bit for bit; that kernel
+// takes the launches of fewer than six elements per SM, whose time is that of a
+// few elements one after the other (us, 512 threads and these: 125 elements 16.3
+// 18.5, 280 24.6 27.3, 800 55.6 56.5, 1728 103.6 100.1, 4352 237 220).
 constexpr int kEight = 8, kEightThreads = 256, kEightBlocks = 13;
 constexpr size_t kEightSmem = kEightBlocks * (sizeof(double) * 512 + sizeof(short) * 64);
 
@@ -288,19 +292,21 @@ cudaError_t launch_kernel(ElemRange r, int nf, const DeviceGeometry &geo, const 
 
 template <int NQ>
 cudaError_t launch_nq(ElemRange r, int nf, const DeviceGeometry &geo, const NativeParams &P,
-                      const FixedTables<16, 4> &fix, const double *q, double *rhs, cudaStream_t s) {
+                      const FixedTables<16, 4> &fix, const double *q, double *rhs, int num_sms,
+                      cudaStream_t s) {
     if (nf == kFields) {
         if constexpr (NQ == kEight) {
-            const cudaError_t e = cudaFuncSetAttribute(vol_rhs_fp64_eight_kernel,
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       (int)kEightSmem);
-            if (e != cudaSuccess) return e;
-            vol_rhs_fp64_eight_kernel<<<(unsigned)r.count, kEightThreads, kEightSmem, s>>>(
-                geo, P, fix, q, rhs, r.M, r.e0);
-            return cudaGetLastError();
-        } else {
-            return launch_kernel<NQ, false>(r, nf, geo, P, fix, q, rhs, s);
+            if (r.count >= 6 * (int64_t)num_sms) {
+                const cudaError_t e = cudaFuncSetAttribute(vol_rhs_fp64_eight_kernel,
+                                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                           (int)kEightSmem);
+                if (e != cudaSuccess) return e;
+                vol_rhs_fp64_eight_kernel<<<(unsigned)r.count, kEightThreads, kEightSmem, s>>>(
+                    geo, P, fix, q, rhs, r.M, r.e0);
+                return cudaGetLastError();
+            }
         }
+        return launch_kernel<NQ, false>(r, nf, geo, P, fix, q, rhs, s);
     }
     return launch_kernel<NQ, true>(r, nf, geo, P, fix, q, rhs, s);
 }
@@ -327,17 +333,17 @@ cudaError_t launch_reference_eos(const double *theta_ref, double *w, double *A, 
 
 cudaError_t launch_vol_rhs_fp64(int N, int nf, ElemRange r, const DeviceGeometry &geo,
                                 const NativeParams &P, const FixedTables<16, 4> &fix,
-                                const double *q, double *rhs, cudaStream_t s) {
+                                const double *q, double *rhs, int num_sms, cudaStream_t s) {
     if (r.count <= 0) return cudaSuccess;
     if (nf < kFields || nf > kMaxFields) return cudaErrorInvalidValue;
     switch (N) {
-        case 1: return launch_nq<2>(r, nf, geo, P, fix, q, rhs, s);
-        case 2: return launch_nq<3>(r, nf, geo, P, fix, q, rhs, s);
-        case 3: return launch_nq<4>(r, nf, geo, P, fix, q, rhs, s);
-        case 4: return launch_nq<5>(r, nf, geo, P, fix, q, rhs, s);
-        case 5: return launch_nq<6>(r, nf, geo, P, fix, q, rhs, s);
-        case 6: return launch_nq<7>(r, nf, geo, P, fix, q, rhs, s);
-        case 7: return launch_nq<8>(r, nf, geo, P, fix, q, rhs, s);
+        case 1: return launch_nq<2>(r, nf, geo, P, fix, q, rhs, num_sms, s);
+        case 2: return launch_nq<3>(r, nf, geo, P, fix, q, rhs, num_sms, s);
+        case 3: return launch_nq<4>(r, nf, geo, P, fix, q, rhs, num_sms, s);
+        case 4: return launch_nq<5>(r, nf, geo, P, fix, q, rhs, num_sms, s);
+        case 5: return launch_nq<6>(r, nf, geo, P, fix, q, rhs, num_sms, s);
+        case 6: return launch_nq<7>(r, nf, geo, P, fix, q, rhs, num_sms, s);
+        case 7: return launch_nq<8>(r, nf, geo, P, fix, q, rhs, num_sms, s);
         default: return cudaErrorInvalidValue;
     }
 }
