@@ -52,6 +52,12 @@ def flops_per_node_fp64(Nq: int) -> int:
     return 5 + 51 + 30 * Nq + 8
 
 
+# What the native FP64 kernel (N = 2..7) issues on the FP64 pipe per point, an FMA
+# as 2: 24 FMAs and 23 other operations; its D sums run in 64-bit fixed point
+# on the integer pipes.
+FP64_PIPE_FLOPS_NATIVE = 71
+
+
 # FP64 CUDA-core peak of one GB300, used only when the FP64 pipe binds: the
 # unit-count figure, and the rate a DFMA microbenchmark measured on the pool.
 FP64_PEAK_TFLOPS = 1.25
@@ -407,13 +413,16 @@ def roofline_entries(kname, kernel_ms, w):
            "bytes_per_point": bpp, "peak_source": peak_src, "kernel_ms": kernel_ms}
     if "mixed" in kname:
         return hbm, None
-    fp64_tfs = flops_per_node_fp64(w.N + 1) * w.M / (kernel_ms * 1e-3) / 1e12
-    # FP64-equivalent flop rate against the FP64 pipe of one GB300 (152 SMs x
+    native = kname.startswith("vol_rhs_fp64")
+    flops = FP64_PIPE_FLOPS_NATIVE if native else flops_per_node_fp64(w.N + 1)
+    fp64_tfs = flops * w.M / (kernel_ms * 1e-3) / 1e12
+    # FP64 flop rate (the native kernel: what it issues on the FP64 pipe; the
+    # double-float kernel: the FP64 operation's equivalent) against the FP64 pipe of one GB300 (152 SMs x
     # 2 DFMA/clk x 2 flop x 2.07 GHz = 1.26 TFLOP/s nominal).  It binds the
     # native kernel; the double-float kernel runs on the FP32 pipes.
     alu = {"bound": "alu", "achieved": fp64_tfs, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
            "frac": fp64_tfs / FP64_PEAK_TFLOPS, "traffic": load_traffic(kname), "kernel": kname,
-           "flops_per_point": flops_per_node_fp64(w.N + 1),
+           "flops_per_point": flops, "algorithmic_flops_per_point": flops_per_node_fp64(w.N + 1),
            "peak_source": "FP64 pipe of one GB300 from its unit counts and clock: 152 SMs x 2 "
                           "DFMA/clk x 2 flop x 2.07 GHz = 1.26, quoted as the nominal 1.25 TFLOP/s",
            "peak_measured_dfma": FP64_DFMA_MEASURED_TFLOPS,
@@ -421,7 +430,7 @@ def roofline_entries(kname, kernel_ms, w):
            "peak_measured_source": "FMA-chain microbenchmark on this pool's GB300 (8 independent "
                                    "DFMA chains per thread): 528 G DFMA/s",
            "kernel_ms": kernel_ms}
-    return (alu, hbm) if kname.startswith("vol_rhs_fp64") else (hbm, alu)
+    return (alu, hbm) if native else (hbm, alu)
 
 
 _ORACLE_RHS = {}

@@ -219,8 +219,9 @@ void numa_vol_destroy(numa_vol *h);
 
 /* Name of the kernel numa_vol_rhs launches for this handle:
  * "vol_rhs_fp64_kernel<Nq>" (NUMA_FP64, or NUMA_DF64 after a geometry
- * fallback), "vol_rhs_df64_kernel" or "vol_rhs_mixed_kernel<Nq>".  Static
- * string; "" for a NULL handle. */
+ * fallback), "vol_rhs_df64_kernel<Nq>", "vol_rhs_mixed_kernel<Nq>" or
+ * "vol_rhs_high_kernel<Nq, type>" (the kernel's name without the forms that a
+ * launch's size chooses among).  Static string; "" for a NULL handle. */
 const char *numa_vol_kernel_name(const numa_vol *h);
 
 /*
@@ -335,7 +336,9 @@ typedef struct {
                                   is set or autotuned */
     int sweep[9];              /* NUMA_SWEEP_CUDA_CORES or NUMA_SWEEP_TENSOR_TF32 */
     int ctas_per_sm;           /* CTAs per SM of the persistent grid: 1 .. 2
-                                  (NUMA_MIXED) or 1 (NUMA_FP64); 0 = the most */
+                                  (NUMA_MIXED); NUMA_FP64 has one grid (two CTAs
+                                  per SM, one with tracers) and takes 1; 0 = the
+                                  most */
     int costliest_first;       /* nonzero: work items sorted by points, largest
                                   first (else instance by instance) */
     int state_in_tmem;         /* NUMA_MIXED, nonzero (the default): the
@@ -535,7 +538,7 @@ void numa_engine_destroy(numa_engine *e);
  * numa_batch of those handles without autotuning.
  *
  * Scratch: the work counter and the instance table live in one fixed __device__
- * array of the library (about 57 KB, held by every GPU that loads the library
+ * array of the library (about 64 KB, held by every GPU that loads the library
  * until the process exits).  The first call on a device does a one-time
  * set-up there: it looks up the array's device address and sets the kernel's
  * shared-memory limit.  Every call overwrites the same array, so calls whose

@@ -39,7 +39,7 @@ constexpr size_t kCounterBytes = 256;
 constexpr size_t kScratchBytes = kCounterBytes + (sizeof(NoallocTable) + 255) / 256 * 256;
 
 // The only device memory this entry point uses.  Every GPU that loads the
-// library holds it (about 57 KB) until the process exits.  Host code never
+// library holds it (about 64 KB) until the process exits.  Host code never
 // dereferences this name: it stands in for the device address, which
 // setup() obtains with cudaGetSymbolAddress.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
