@@ -506,7 +506,7 @@ cudaError_t launch_high_form(ElemRange r, int nf, const Geo &geo, const Params &
     cudaError_t e = cudaFuncSetAttribute(vol_rhs_high_kernel<NQ, T, NF>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    int64_t ahead = 0;   // FP64: no prefetch (bound by the FP64 pipe)
+    int64_t ahead = 0;   // FP64: no prefetch (not measured since the sweeps left the FP64 pipe)
     if (sizeof(T) == 4 && num_sms > 0) {
         int per_sm = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, vol_rhs_high_kernel<NQ, T, NF>,
