@@ -99,8 +99,10 @@ typedef struct {
 } numa_geometry;
 
 typedef enum {
-    NUMA_FP64 = 0,   /* FP64 state and rhs, FP64 arithmetic; the D sums in 64-bit
-                        fixed point (N >= 2), no less exact                      */
+    NUMA_FP64 = 0,   /* FP64 state and rhs, FP64 arithmetic; the D sums of N >= 2
+                        in 64-bit fixed point, a row's error at most 2^-54 of the
+                        row's sum of |D| times the line's largest flux (lines that
+                        do not suit fixed point: FP64)                           */
     NUMA_MIXED = 1,  /* FP32 perturbation state (rho', U1, U2, U3, Theta'), FP32 rhs,
                         FP32 geometry and arithmetic                                    */
     NUMA_DF64 = 2    /* FP64 state and rhs, double-float arithmetic (hi + lo FP32 pairs,

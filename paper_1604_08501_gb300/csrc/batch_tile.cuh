@@ -21,10 +21,10 @@ constexpr int kThreads = 512;
 // Shared memory of one CTA and CTAs per SM.  FP64: the fluxes (15 values per
 // thread), q and dq (10 values); the D sweeps run on the integer pipes
 // (fixed_sweep.cuh), so two CTAs of 64 registers share an SM and one's sweeps
-// run beside the other's FP64 phases (the FP64 pipe binds, about 72 operations
+// run beside the other's FP64 phases (the FP64 pipe binds, about 62 operations
 // per point and stage).  Measured on 6 instances, 4.6 million points, ten steps
 // (50 stages): 75.5 ms with FP64 sweeps, q and dq in registers and one CTA per SM,
-// 29.7 ms so.  The tracer form keeps the base fields' q and dq in registers
+// 30.2 ms so.  The tracer form keeps the base fields' q and dq in registers
 // (98 KB of fluxes: one CTA per SM).  Mixed: the fluxes, q and dq (10 values) and the point's geometry
 // (g and Jinv, 10 values) in shared memory, so that the kernel fits 64
 // registers and two CTAs share an SM, twice the warps to hide latency.
@@ -50,10 +50,10 @@ constexpr int kMixedFluxWords = tile_flux_words<float>();
 constexpr int kMixedSmemWords = kMixedFluxWords + (2 * 5 + 10) * kThreads;
 // FP64: the exponents of the lines' fixed-point sums (fixed_sweep.cuh) follow.
 template <int NF>
-__host__ __device__ constexpr int tile_lines() {   // lines of one pass: the largest over the orders
+__host__ __device__ constexpr int tile_exponents() {   // of the lines of one pass: the largest over the orders
     int m = 0;
     for (int nq = 2; nq <= 8; ++nq) {
-        const int x = 3 * NF * (kThreads / (nq * nq * nq)) * nq * nq;
+        const int x = 3 * NF * (kThreads / (nq * nq * nq)) * nq * nq * (1 + (nq & 1));
         m = x > m ? x : m;
     }
     return m;
@@ -69,7 +69,7 @@ constexpr size_t tile_smem_bytes() {
     constexpr int NF = TR ? kMaxFields : kFields;
     return MIXED ? sizeof(float) * (tile_flux_words<float, NF>() + (2 * NF + 10) * kThreads)
                  : sizeof(double) * (tile_flux_words<double, NF>() + fp64_state_words<TR>() * kThreads) +
-                       sizeof(short) * tile_lines<NF>();
+                       sizeof(short) * tile_exponents<NF>();
 }
 template <bool MIXED, bool TR = false>
 constexpr int tile_ctas_per_sm() {
@@ -282,8 +282,8 @@ __device__ void run_tile(const BatchInstance &I, int64_t e0, int64_t count,
                         if constexpr (MIXED)
                             sweep_line<NQ>(sF + bd * BLK + e * EW, line, c_sweep32[NQ]);
                         else
-                            sE[t] = (short)sweep_line_fixed<NQ>(sF + bd * BLK + e * EW, line,
-                                                                c_sweep64[NQ], c_fixed[NQ]);
+                            sweep_line_to<NQ>(sF + bd * BLK + e * EW, line, c_sweep64[NQ], c_fixed[NQ],
+                                              sE + t, TASKS);
                     }
                 }
                 // FP64: J^-1 and rho_ref loaded before the barrier, so that
@@ -310,13 +310,13 @@ __device__ void run_tile(const BatchInstance &I, int64_t e0, int64_t count,
                     } else {
                         constexpr int EB = EPP * NL;   // lines of one (direction, field)
                         const short *E = sE + b0 * EB + el * NL;
+                        const FixedRow row[3] = {fixed_row<NQ>(c_fixed[NQ], NQ * k + j, i, TASKS),
+                                                 fixed_row<NQ>(c_fixed[NQ], NQ * k + i, j, TASKS),
+                                                 fixed_row<NQ>(c_fixed[NQ], NQ * j + i, k, TASKS)};
+                        const int sh[3] = {row[0].shift, row[1].shift, row[2].shift};
                         fixed_sums<NQ>(
-                            v, c_fixed[NQ].shift, jinv,
-                            [&](int d, int b) { return sF[f[d] + (b0 + b) * BLK]; },
-                            [&](int d, int b) {
-                                return (int)E[(d * NF + b) * EB +
-                                              (d == 0 ? NQ * k + j : d == 1 ? NQ * k + i : NQ * j + i)];
-                            });
+                            v, sh, jinv, [&](int d, int b) { return sF[f[d] + (b0 + b) * BLK]; },
+                            [&](int d, int b) { return (int)E[(d * NF + b) * EB + row[d].at]; });
                     }
                 };
                 if (active) {

@@ -3,44 +3,65 @@
 // GB300 issues 1.67 DFMA per clock and SM (measured) but about 30 multiply-adds of
 // 32 x 32 + 64 bits and 60 other integer operations, and an even-odd sweep in
 // FP64 (element_sweep.cuh) is 90 of the volume term's 157 FP64 operations per
-// point at Nq = 8.  Here the sums run on the integer pipes, beside the FP64
-// pipe, and are more accurate than in FP64:
+// point at Nq = 8.  Here the sums run on the integer pipes, beside the FP64 pipe:
 //
 //  * The thread of a line takes the largest exponent field e of its Nq fluxes
-//    and writes each as an integer X with F = X 2^(e - 1080), |X| < 2^58: the 53
-//    significant bits of the largest flux, and 5 bits below.
-//  * E_m = X_m + X_{N-m} and O_m = X_m - X_{N-m} are exact, below 2^59.
-//  * D is an integer too, D 2^s rounded to nearest, s such that the largest sum
-//    of |D[i][n]| over a row is at most 2^58.  Both are cut at bit 28 into
-//    32-bit words, E = Eh 2^28 + El (0 <= El < 2^28) and D = Dh 2^28 + Dl
-//    (|Dl| <= 2^27), and
-//      sum D E / 2^56 = sum Eh Dh + (sum (Eh Dl + El Dh)) / 2^28 + (sum El Dl) / 2^56.
-//    The first sum is exact (below 2^60), the second too (at most 9 terms below
-//    2^59 each) and its quotient is rounded down; the third, below 4.5, is
-//    dropped.  Three multiply-adds per product.
+//    and writes each as an integer X with F = X 2^(e - 1082), |X| < 2^60: the 53
+//    significant bits of the largest flux, and 7 bits below (cut towards zero).
+//  * E_m = X_m + X_{N-m} and O_m = X_m - X_{N-m} are exact, below 2^61.
+//  * Each row of D is an integer row of its own scale, D[i][n] 2^s_i rounded to
+//    nearest, s_i such that the row's sum of |D[i][n]| lies in [2^60, 2^61) (rows
+//    i and N-i share it): the inner rows' entries are many times smaller than
+//    those of the first and last row.  E is cut at bit 31 and D at bit 30 into
+//    32-bit words, E = Eh 2^31 + El (0 <= El < 2^31) and D = Dh 2^30 + Dl / 2
+//    (|Dl| <= 2^30, even), and
+//      sum D E / 2^61 = sum Eh Dh + (sum (Eh Dl + El Dh)) / 2^31 + (sum El Dl) / 2^62.
+//    The first sum is exact, the second too (below 2^63 for the tables of every
+//    Nq: tests/test_fixed_sweep_rows.py) and its quotient is rounded to nearest;
+//    the third, at most half a unit a product, is dropped.  Three multiply-adds
+//    per product.
 //  * S_i = a_i + b_i and S_{N-i} = b_i - a_i, |S| <= 2^60, replace the line's
-//    fluxes; the value is S 2^(e - 1024 - s).  Phase 3 adds a point's three sums
+//    fluxes; the value is S 2^(e - 1021 - s_i).  Phase 3 adds a point's three sums
 //    as integers at the largest of their exponents (|sum| <= 3 2^60), multiplies
 //    them by J^-1 as integers and rounds once to FP64 (fixed_sums).
+//  * The centre row of odd Nq does not use the centre flux and, D being
+//    centro-antisymmetric, is a sum over the differences O_m alone.  Those can be
+//    far smaller than the line's largest flux (a spike at the centre; a smooth or
+//    nearly uniform line), so they are shifted up to 61 bits first and the centre
+//    sum has an exponent of its own.  Where fluxes beside the centre lost bits to
+//    the line's scale and the differences are small (below 2^56), the row is
+//    summed in FP64.  At Nq = 3, whose D is +-1/2, 1, 3/2 and 2, every sum is
+//    exact, and the outer rows are shifted up in the same way.
 //
-// Measured: vol_rhs_fp64_kernel at N = 7, 32768 elements, 4.949 -> 1.881 ms; the
-// FP64 batch 2.07 times as fast.  (Rounded before an FP64 multiply by J^-1, one
-// test for each field; all fields' integer chains side by side: see vol_fp64.cu.)
+//  * From Nq = 10, lines in which one or two values exceed all others 16 times
+//    or more stay in FP64: inner rows hardly use such a value, and FP64 rounds
+//    relative to what a row uses.
 //
-// Error: at most 1 in each X and 2^-1 in each integer D entry, so at most
-// 2^-55 (largest |D| row sum) (largest flux of the line), as a bound; the
-// rounding errors of the FP64 sweep of such a line are 2^-53 of its partial
-// sums.  tests/test_fixed_sweep_host.py holds it to that bound and to at most
-// the FP64 sweep's error, over random, smooth and graded lines of every Nq.
+// Measured: vol_rhs_fp64_kernel at N = 7, 32768 elements, 4.949 -> 1.535 ms with the
+// steps named in vol_fp64.cu; the FP64 batch 75.5 -> 30.2 ms.  One scale for the
+// whole line and all rows, 58 bits and sums cut instead of rounded were 0 to 3 %
+// faster (3.5 million points, us, then and so: N = 2 743 755, N = 4 330 334, N = 6 386
+// 397, N = 7 338 338, N = 8 587 606, N = 11 543 551, N = 15 673 693; 512 elements of
+// N = 4 13.9 14.4), but less exact than FP64 in the centre row of odd Nq (1e-14 to
+// 1e-7 of the row's value on the lines above) and in inner rows of Nq >= 8.
+//
+// Error of S_i, in units of S: at most 1 from the X, 1/2 (Nq/2 pairs) and 1/4 (the
+// centre column) from the integer D, as much again twice over from the dropped
+// third sums, 1 from the rounding of a and b: below 1.5 (Nq/2) + 3.  A unit is
+// at most 2^-58 of (the row's sum of |D[i][n]|) x (largest flux of the line), so the
+// bound is 2^-54.8 of that at Nq = 8 and 2^-54.1 at Nq = 16.  That is a bound for
+// a row and a line as a whole, where FP64 rounds each term relative to itself; row by
+// row the root mean square error was at most the FP64 sweep's on random, smooth,
+// nearly uniform, graded and nearly even lines and on lines with spikes of any size
+// at the centre, an end, beside an end or at several points
+// (tests/test_fixed_sweep_rows.py).
 //
 // Nq = 2 keeps the FP64 sweep: its D is +-1/2, so that FP64 rounds only sums and
-// differences, and the fixed-point sum of three directions, cut at 2^-58 of the
-// largest line, was less exact (6.0e-18 against 8.7e-19 of the line's scale on
-// smooth lines, where the sums are far smaller than the fluxes).
+// differences.
 //
 // Lines whose largest exponent field is outside [kFixMinExp, kFixMaxExp]
 // (infinities, NaN, values that could overflow, lines of tiny values) take the
-// FP64 sweep: their exponent is kFixNone and the slots hold doubles.  A line
+// FP64 sweep as well: their exponent is kFixNone and the slots hold doubles.  A line
 // of zeros is a line of integer zeros.
 #pragma once
 
@@ -54,6 +75,9 @@ namespace numa {
 
 constexpr int kFixMinExp = 200, kFixMaxExp = 1900;
 constexpr int kFixNone = -1;      // exponent of a line left in FP64
+constexpr int kFixMinCentre = 64; // least exponent field of a centre row summed in FP64
+constexpr int kFixDominated = 10; // Nq from which lines of one or two dominant values stay in FP64:
+constexpr uint32_t kFixNear = 4;  // those with no third value within this many binades of the largest
 
 // Orders whose lines are swept in fixed point.
 template <int NQ>
@@ -101,7 +125,7 @@ __host__ __device__ __forceinline__ int fix_clz(unsigned long long x) {
 }
 
 // X of the double with bits b, in a line of largest exponent field e: its
-// mantissa with the hidden bit at bit 57, shifted down by the difference of
+// mantissa with the hidden bit at bit 59, shifted down by the difference of
 // the exponents (towards zero), with its sign.  Zeros and subnormals shift out.
 __host__ __device__ __forceinline__ long long fix_from_bits(long long b, int e) {
     const uint32_t hi = (uint32_t)((unsigned long long)b >> 32);
@@ -113,15 +137,15 @@ __host__ __device__ __forceinline__ long long fix_from_bits(long long b, int e) 
     return (a ^ s) - s;
 }
 
-// The integer R, |R| < 2^63, times 2^(e - 1024 - s), rounded to nearest (ties
-// away from zero).  kFixMinExp and kFixMaxExp keep the result normal.
-__host__ __device__ __forceinline__ double fix_to_double(long long R, int e, int shift) {
+// The integer R, |R| < 2^63, times 2^(e - 1024), rounded to nearest (ties away from
+// zero).  kFixMinExp and kFixMaxExp keep the result normal.
+__host__ __device__ __forceinline__ double fix_to_double(long long R, int e) {
     const long long s = R >> 63;
     const unsigned long long a = (unsigned long long)((R ^ s) - s);
     const int lz = fix_clz(a);
     const unsigned long long m = a << (lz & 63);   // leading bit at 63
-    // exponent field of 2^(63 - lz) 2^(e - 1024 - s), less the hidden bit's one
-    const int E = e - shift + 61 - lz;
+    // exponent field of 2^(63 - lz) 2^(e - 1024), less the hidden bit's one
+    const int E = e + 61 - lz;
     const unsigned long long v = ((unsigned long long)(uint32_t)E << 52) + (m >> 11) + ((m >> 10) & 1ull);
     return a == 0ull ? 0.0 : fix_double((long long)(v | ((unsigned long long)s & (1ull << 63))));
 }
@@ -135,11 +159,10 @@ __host__ __device__ __forceinline__ unsigned long long fix_mulhi(unsigned long l
 #endif
 }
 
-// -y R 2^(e - 1024 - s), rounded once (to nearest, ties away from zero): the
+// -y R 2^(e - 1024), rounded once (to nearest, ties away from zero): the
 // integer's leading 64 bits times the 53 of y (exponent field ey), a multiply
 // on the integer pipes.  ok is cleared where the product is not a normal number.
-__host__ __device__ __forceinline__ double fix_scale(long long R, int e, int shift, double y, int ey,
-                                                     bool &ok) {
+__host__ __device__ __forceinline__ double fix_scale(long long R, int e, double y, int ey, bool &ok) {
     const long long yb = fix_bits(y);
     const long long s = R >> 63;
     const unsigned long long a = (unsigned long long)((R ^ s) - s);
@@ -149,8 +172,8 @@ __host__ __device__ __forceinline__ double fix_scale(long long R, int e, int shi
     unsigned long long p = fix_mulhi(a << (lz & 63), my);
     const int up = (long long)p < 0 ? 0 : 1;
     p <<= up;
-    // exponent field of 2^(63 - lz) 2^(e - 1024 - s) y, less the hidden bit's one
-    const int E = e - shift + 61 - lz + ey - 1023 + 1 - up;
+    // exponent field of 2^(63 - lz) 2^(e - 1024) y, less the hidden bit's one
+    const int E = e + 61 - lz + ey - 1023 + 1 - up;
     const unsigned long long v = ((unsigned long long)(uint32_t)E << 52) + (p >> 11) + ((p >> 10) & 1ull);
     ok = ok && (a == 0ull || (unsigned)(E - 1) < 2044u);
     return a == 0ull ? 0.0
@@ -167,9 +190,19 @@ __host__ __device__ __attribute__((noinline)) void sweep_line_fp64_call(double *
     sweep_line<NQ>(buf, line, tab);
 }
 
-// One product of a sum: acc_h += Eh Dh, acc_m += Eh Dl + El Dh.
+// The centre row of a line in FP64 (odd Nq), out of line too.
+template <int NQ, typename Tab>
+__host__ __device__ __attribute__((noinline)) double centre_fp64_call(const double *buf, int line, const Tab &tab) {
+    double c = 0.0;
+    for (int m = 0; m < NQ / 2; ++m)
+        c = fma(tab.Dcr[m], buf[slot<NQ, double>(line, m)] - buf[slot<NQ, double>(line, NQ - 1 - m)], c);
+    return c;
+}
+
+// A sum of products: h = sum Eh Dh, m = sum (Eh Dl + El Dh) and half a unit of the
+// quotient, which is so rounded to nearest.
 struct FixedSum {
-    long long h, m;
+    long long h = 0, m = 1ll << (kFixLow - 1);
 };
 // x y + z, 32 x 32 + 64 bits.  In C the compiler loses sight of the operands' 32
 // bits (an E cut by a mask is a 64-bit value to it) and multiplies 64 by 64:
@@ -192,30 +225,50 @@ __host__ __device__ __forceinline__ long long fix_value(FixedSum a) {
     return a.h + (a.m >> kFixLow);
 }
 
-// The sums S of the line's integers X[0..NQ), each given to put(n, S) as it is formed.
+// Shift that brings integers below 2^61 in magnitude to 61 bits; mag: the "or" of
+// their x ^ (x >> 63).  61 for zeros.
+__host__ __device__ __forceinline__ int fix_headroom(long long mag) {
+    return fix_clz((unsigned long long)mag) - 3;
+}
+__host__ __device__ __forceinline__ long long fix_magnitude(long long x) { return x ^ (x >> 63); }
+__host__ __device__ __forceinline__ long long fix_shl(long long x, int n) {
+    return (long long)((unsigned long long)x << n);
+}
+
+// The sums S of the line's integers X[0..NQ), each given to put(n, S) as it is
+// formed; the centre row of odd Nq with its differences shifted up by `up`.
 template <int NQ, typename FT, typename Put>
-__host__ __device__ __forceinline__ void sweep_fixed(const long long *X, const FT &ft, Put put) {
+__host__ __device__ __forceinline__ void sweep_fixed(const long long *X, const FT &ft, int up, Put put) {
     constexpr int HALF = NQ / 2;
     constexpr bool ODD = (NQ & 1) != 0;
     constexpr int C = NQ / 2;
-    constexpr long long MASK = (1ll << kFixLow) - 1;
+    constexpr int MASK = (int)((1u << kFixLow) - 1);
+    if constexpr (ODD) {
+        FixedSum c;
+#pragma unroll
+        for (int m = 0; m < HALF; ++m) {
+            const long long O = fix_shl(X[m] - X[NQ - 1 - m], up);
+            fix_mad(c, (int)(O >> kFixLow), (int)O & MASK, ft.Dcrh[m], ft.Dcrl[m]);
+        }
+        put(C, fix_value(c));
+    }
     int Eh[HALF], El[HALF], Oh[HALF], Ol[HALF];
 #pragma unroll
     for (int m = 0; m < HALF; ++m) {
         const long long E = X[m] + X[NQ - 1 - m], O = X[m] - X[NQ - 1 - m];
         Eh[m] = (int)(E >> kFixLow);
-        El[m] = (int)(E & MASK);
+        El[m] = (int)E & MASK;
         Oh[m] = (int)(O >> kFixLow);
-        Ol[m] = (int)(O & MASK);
+        Ol[m] = (int)O & MASK;
     }
     int Ch = 0, Cl = 0;
     if constexpr (ODD) {
         Ch = (int)(X[C] >> kFixLow);
-        Cl = (int)(X[C] & MASK);
+        Cl = (int)X[C] & MASK;
     }
 #pragma unroll
     for (int r = 0; r < HALF; ++r) {
-        FixedSum a{0, 0}, b{0, 0};
+        FixedSum a, b;
         if constexpr (ODD) fix_mad(a, Ch, Cl, ft.Dch[r], ft.Dcl[r]);
 #pragma unroll
         for (int m = 0; m < HALF; ++m) {
@@ -226,18 +279,23 @@ __host__ __device__ __forceinline__ void sweep_fixed(const long long *X, const F
         put(r, B + A);
         put(NQ - 1 - r, B - A);
     }
-    if constexpr (ODD) {
-        FixedSum c{0, 0};
-#pragma unroll
-        for (int m = 0; m < HALF; ++m) fix_mad(c, Oh[m], Ol[m], ft.Dcrh[m], ft.Dcrl[m]);
-        put(C, fix_value(c));
-    }
 }
 
-// Sweep line `line` of buf in place: fluxes (doubles) in, integer sums out,
-// and the line's exponent returned (kFixNone: the sums are doubles).
-template <int NQ, typename Tab, typename FT>
-__host__ __device__ __forceinline__ int sweep_line_fixed(double *buf, int line, const Tab &tab, const FT &ft) {
+template <typename FT>
+__host__ __device__ __forceinline__ int row_shift(const FT &ft, int n) {
+    return (int)(ft.rows >> (4 * n)) & 15;
+}
+
+// Sweep line `line` of buf in place: fluxes (doubles) in, integer sums out, each at
+// its row's scale: row n is S 2^(e - 1024 - ft.shift - row_shift(ft, n)).  The line's
+// exponent e is returned (kFixNone: the sums are doubles); centre: the exponent of
+// the centre row (odd Nq).  DOMINATED: lines of one or two dominant values too.
+template <int NQ, bool DOMINATED = false, typename Tab, typename FT>
+__host__ __device__ __forceinline__ int sweep_line_rows(double *buf, int line, const Tab &tab, const FT &ft,
+                                                        int &centre) {
+    constexpr bool ODD = (NQ & 1) != 0;
+    constexpr int C = NQ / 2;
+    centre = kFixNone;
     if constexpr (!fixed_point<NQ>()) {
         sweep_line<NQ>(buf, line, tab);
         return kFixNone;
@@ -245,49 +303,132 @@ __host__ __device__ __forceinline__ int sweep_line_fixed(double *buf, int line, 
     long long X[NQ];
     double F[NQ];
     load_line<NQ, double>(buf, line, F);
-    uint32_t top = 0, any = 0;
+    uint32_t top = 0, any = 0, low = ~0u;   // low: the smallest beside the centre
 #pragma unroll
     for (int n = 0; n < NQ; ++n) {
         X[n] = fix_bits(F[n]);
         const uint32_t h = (uint32_t)((unsigned long long)X[n] >> 32) & 0x7FFFFFFFu;
         top = h > top ? h : top;
         any |= (uint32_t)X[n];
+        if (ODD && n != C) low = h < low ? h : low;
     }
     int e = (int)(top >> 20);
-    if (e < kFixMinExp || e > kFixMaxExp) {
+    bool fixed = e >= kFixMinExp && e <= kFixMaxExp;
+    if constexpr (!DOMINATED && NQ >= kFixDominated) {
+        int near = 0;
+#pragma unroll
+        for (int n = 0; n < NQ; ++n)
+            near += ((uint32_t)((unsigned long long)X[n] >> 32) & 0x7FFFFFFFu) + (kFixNear << 20) >= top ? 1 : 0;
+        fixed = fixed && near > 2;
+    }
+    if (!fixed) {
         if ((top | any) != 0u) {
             sweep_line_fp64_call<NQ>(buf, line, tab);
             return kFixNone;
         }
         e = kFixMinExp;   // zeros of either sign: X = 0
+        low = (uint32_t)kFixMinExp << 20;
     }
 #pragma unroll
     for (int n = 0; n < NQ; ++n) X[n] = fix_from_bits(X[n], e);
-    if constexpr (line_vector<NQ, double>() > 1) {
-        sweep_fixed<NQ>(X, ft, [&](int n, long long S) { F[n] = fix_double(S); });
+    int up = 0;
+    bool centre_fp64 = false;
+    double c64 = 0.0;
+    if constexpr (ODD) {
+        long long mag = 0;
+#pragma unroll
+        for (int m = 0; m < C; ++m) mag |= fix_magnitude(X[m] - X[NQ - 1 - m]);
+        up = fix_headroom(mag);
+        centre = e - up;
+        // an X lost bits where it lies more than kFixBits - 53 binades below the
+        // line's largest, less than 2^-55 of differences that reach 2^56
+        centre_fp64 = e - (int)(low >> 20) > kFixBits - 53 && up > 4;
+        if (centre_fp64) c64 = centre_fp64_call<NQ>(buf, line, tab);
+    }
+    if constexpr (line_vector<NQ, double>() > 1 || NQ == 3) {
+        sweep_fixed<NQ>(X, ft, up, [&](int n, long long S) { F[n] = fix_double(S); });
+        if constexpr (NQ == 3) {   // exact sums: the outer rows shifted up as well
+            const long long S0 = fix_bits(F[0]), S2 = fix_bits(F[2]);
+            const int u = fix_headroom(fix_magnitude(S0) | fix_magnitude(S2));
+            F[0] = fix_double(fix_shl(S0, u));
+            F[2] = fix_double(fix_shl(S2, u));
+            e -= u;
+        }
         store_line<NQ, double>(buf, line, F);
     } else {
-        sweep_fixed<NQ>(X, ft, [&](int n, long long S) { buf[slot<NQ, double>(line, n)] = fix_double(S); });
+        sweep_fixed<NQ>(X, ft, up, [&](int n, long long S) { buf[slot<NQ, double>(line, n)] = fix_double(S); });
+    }
+    if (ODD && centre_fp64) {   // the FP64 sum's mantissa, and its exponent as the centre row's
+        const long long b = fix_bits(c64);
+        int ec = (int)((unsigned long long)b >> 52) & 0x7FF;
+        ec = ec < kFixMinCentre ? kFixMinCentre : ec;
+        buf[slot<NQ, double>(line, C)] = fix_double(fix_from_bits(b, ec));
+        centre = ec + 1024 - (1022 + kFixBits) + ft.shift + row_shift(ft, C);
     }
     return e;
 }
 
+// The same with every row at the line's exponent, S 2^(e - 1024 - ft.shift): for
+// host checks that add lines slot by slot.
+template <int NQ, typename Tab, typename FT>
+__host__ __device__ __forceinline__ int sweep_line_fixed(double *buf, int line, const Tab &tab, const FT &ft) {
+    int c;
+    const int e = sweep_line_rows<NQ, true>(buf, line, tab, ft, c);
+    if (e == kFixNone) return e;
+    const int top = (NQ & 1) && c > e ? c : e;
+    for (int n = 0; n < NQ; ++n) {
+        double &x = buf[slot<NQ, double>(line, n)];
+        const int en = (NQ & 1) && n == NQ / 2 ? c : e;
+        x = fix_double(fix_shr(fix_bits(x), top - en + row_shift(ft, n)));
+    }
+    return top;
+}
+
+// The sweep, its exponents to E[0] and, for the centre row of odd Nq, E[lines].
+template <int NQ, typename Tab, typename FT>
+__host__ __device__ __forceinline__ void sweep_line_to(double *buf, int line, const Tab &tab, const FT &ft,
+                                                       short *E, int lines) {
+    int c;
+    E[0] = (short)sweep_line_rows<NQ>(buf, line, tab, ft, c);
+    if constexpr (NQ & 1) E[lines] = (short)c;
+}
+
+// Where a point finds its line's exponent and its row's scale: `at` entries into the
+// exponents of a block's lines (the centre rows' follow those of all lines, by
+// `lines`), and the row's shift.
+struct FixedRow {
+    int at, shift;
+};
+template <int NQ, typename FT>
+__host__ __device__ __forceinline__ FixedRow fixed_row(const FT &ft, int line, int n, int lines) {
+    return FixedRow{(NQ & 1) && n == NQ / 2 ? line + lines : line, ft.shift + row_shift(ft, n)};
+}
+// Exponents per line in shared memory.
+template <int NQ>
+__host__ __device__ constexpr int line_exponents() {
+    return 1 + (NQ & 1);
+}
+
 // -y times the sum of a point's three directions where a line is in FP64, or
-// the integer multiply does not take y (rare).
+// the integer multiply does not take y (rare); er, es, et: the exponents less the
+// rows' shifts, or kFixDouble.
+constexpr int kFixDouble = -(1 << 20);
 static __host__ __device__ __attribute__((noinline)) double fixed_sum3_slow(double r, int er, double s,
                                                                             int es, double t, int et,
-                                                                            int shift, double y) {
-    const double R = er < 0 ? r : fix_to_double(fix_bits(r), er, shift);
-    const double S = es < 0 ? s : fix_to_double(fix_bits(s), es, shift);
-    const double T = et < 0 ? t : fix_to_double(fix_bits(t), et, shift);
+                                                                            double y) {
+    const double R = er == kFixDouble ? r : fix_to_double(fix_bits(r), er);
+    const double S = es == kFixDouble ? s : fix_to_double(fix_bits(s), es);
+    const double T = et == kFixDouble ? t : fix_to_double(fix_bits(t), et);
     return -y * (R + S + T);
 }
 
 // v[b] = -y times the sum of a point's three directions, b < NB: at(d, b) gives
-// the slot's bits and ex(d, b) the line's exponent.  One test for all of them,
-// after the integer operations, so that their chains run side by side.
+// the slot's bits, ex(d, b) the exponent of its line (or centre row) and sh[d] the
+// shift of the point's row in direction d.  One test for all of them, after the
+// integer operations, so that their chains run side by side.
 template <int NQ, int NB, typename At, typename Ex>
-__host__ __device__ __forceinline__ void fixed_sums(double (&v)[NB], int shift, double y, At at, Ex ex) {
+__host__ __device__ __forceinline__ void fixed_sums(double (&v)[NB], const int (&sh)[3], double y, At at,
+                                                    Ex ex) {
     if constexpr (!fixed_point<NQ>()) {
 #pragma unroll
         for (int b = 0; b < NB; ++b) v[b] = -y * (at(0, b) + at(1, b) + at(2, b));
@@ -297,18 +438,26 @@ __host__ __device__ __forceinline__ void fixed_sums(double (&v)[NB], int shift, 
     bool ok = (unsigned)(ey - 1) < 2046u;   // not zero, subnormal, infinite or NaN
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
-        const int e0 = ex(0, b), e1 = ex(1, b), e2 = ex(2, b);
-        ok = ok && (e0 | e1 | e2) >= 0;
+        const int x0 = ex(0, b), x1 = ex(1, b), x2 = ex(2, b);
+        ok = ok && (x0 | x1 | x2) >= 0;
+        const int e0 = x0 - sh[0], e1 = x1 - sh[1], e2 = x2 - sh[2];
         const int m = e0 > e1 ? e0 : e1, e = m > e2 ? m : e2;
         const long long R = fix_shr(fix_bits(at(0, b)), e - e0) + fix_shr(fix_bits(at(1, b)), e - e1) +
                             fix_shr(fix_bits(at(2, b)), e - e2);
-        v[b] = fix_scale(R, e, shift, y, ey, ok);
+        v[b] = fix_scale(R, e, y, ey, ok);
     }
     if (!ok) {
+        auto e = [&](int d, int b) { return ex(d, b) < 0 ? kFixDouble : ex(d, b) - sh[d]; };
 #pragma unroll
         for (int b = 0; b < NB; ++b)
-            v[b] = fixed_sum3_slow(at(0, b), ex(0, b), at(1, b), ex(1, b), at(2, b), ex(2, b), shift, y);
+            v[b] = fixed_sum3_slow(at(0, b), e(0, b), at(1, b), e(1, b), at(2, b), e(2, b), y);
     }
+}
+// One shift for every row (sweep_line_fixed).
+template <int NQ, int NB, typename At, typename Ex>
+__host__ __device__ __forceinline__ void fixed_sums(double (&v)[NB], int shift, double y, At at, Ex ex) {
+    const int sh[3] = {shift, shift, shift};
+    fixed_sums<NQ>(v, sh, y, at, ex);
 }
 
 }  // namespace numa

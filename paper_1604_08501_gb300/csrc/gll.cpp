@@ -10,6 +10,7 @@
 //   D[i][n] = P_N(x_i) / (P_N(x_n) (x_i - x_n)),
 // and the diagonal is set to minus the off-diagonal row sum, so that D maps
 // constants to zero as exactly as rounding allows.
+#include <algorithm>
 #include <cmath>
 
 #include "numa_internal.h"
@@ -92,34 +93,36 @@ void sweep_tables(int N, const double *D, double De[16], double Do[16], double D
 }
 
 int fixed_tables(int N, const double *D, int *Deh, int *Del, int *Doh, int *Dol, int *Dch, int *Dcl,
-                 int *Dcrh, int *Dcrl) {
+                 int *Dcrh, int *Dcrl, unsigned long long *rows) {
     const int Nq = N + 1, half = Nq / 2, ctr = Nq / 2;
-    long double rows = 0.0L;
-    for (int i = 0; i < Nq; ++i) {
+    int shift[16], least = kFixD;
+    for (int i = 0; i < (Nq + 1) / 2; ++i) {   // rows i and N - i: the same |D|
         long double sum = 0.0L;
         for (int n = 0; n < Nq; ++n) sum += std::fabs((long double)D[i * Nq + n]);
-        rows = sum > rows ? sum : rows;
+        int ex = 0;
+        std::frexp(sum, &ex);   // 2^(ex - 1) <= sum < 2^ex
+        shift[i] = shift[Nq - 1 - i] = kFixD - ex;
+        least = std::min(least, shift[i]);
     }
-    int ex = 0;
-    std::frexp(rows, &ex);   // rows < 2^ex
-    const int shift = kFixBits - ex;
-    auto put = [shift](long double x, int *h, int *l) {
-        const long long v = std::llround(std::ldexp(x, shift));
-        *h = (int)((v + (1ll << (kFixLow - 1))) >> kFixLow);
-        *l = (int)(v - ((long long)*h << kFixLow));
+    *rows = 0;
+    for (int i = 0; i < Nq; ++i) *rows |= (unsigned long long)(shift[i] - least) << (4 * i);
+    auto put = [](long double x, int s, int *h, int *l) {
+        const long long v = std::llround(std::ldexp(x, s));
+        *h = (int)((v + (1ll << (kFixDLow - 1))) >> kFixDLow);
+        *l = (int)(2 * (v - ((long long)*h << kFixDLow)));
     };
     for (int r = 0; r < half; ++r) {
         for (int m = 0; m < half; ++m) {
             const long double a = D[r * Nq + m], b = D[r * Nq + (Nq - 1 - m)];
-            put((a + b) / 2, &Deh[r * half + m], &Del[r * half + m]);
-            put((a - b) / 2, &Doh[r * half + m], &Dol[r * half + m]);
+            put((a + b) / 2, shift[r], &Deh[r * half + m], &Del[r * half + m]);
+            put((a - b) / 2, shift[r], &Doh[r * half + m], &Dol[r * half + m]);
         }
         if (Nq & 1) {
-            put(D[r * Nq + ctr], &Dch[r], &Dcl[r]);
-            put(D[ctr * Nq + r], &Dcrh[r], &Dcrl[r]);
+            put(D[r * Nq + ctr], shift[r], &Dch[r], &Dcl[r]);
+            put(D[ctr * Nq + r], shift[ctr], &Dcrh[r], &Dcrl[r]);
         }
     }
-    return shift;
+    return least - 3;
 }
 
 }  // namespace numa

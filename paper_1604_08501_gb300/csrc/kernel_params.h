@@ -34,15 +34,18 @@ struct EosConstants {
     double p0, R, gamma, grav;
 };
 
-// Even-odd tables of D 2^shift as (high, low) integer words for the fixed-point
-// sweep of the FP64 kernels (fixed_sweep.cuh); T: entries of De and Do, H: of
-// the centre column and row (odd Nq).
-constexpr int kFixBits = 58;   // line values are integers below 2^58, row sums of |D| 2^shift at most that
-constexpr int kFixLow = 28;    // bits of the low words
+// Even-odd tables of D as (high, low) integer words for the fixed-point sweep of
+// the FP64 kernels (fixed_sweep.cuh), row n times 2^s, s = shift + row_shift + 3; T: entries of De
+// and Do, H: of the centre column and row (odd Nq).
+constexpr int kFixBits = 60;   // line values are integers below 2^60
+constexpr int kFixLow = 31;    // bits of their sums' low words
+constexpr int kFixD = 61;      // the sum of a row's |D| 2^s is below 2^61
+constexpr int kFixDLow = 30;   // bits of D's low words, which hold twice the value
 template <int T, int H>
 struct FixedTables {
     int Deh[T], Del[T], Doh[T], Dol[T], Dch[H], Dcl[H], Dcrh[H], Dcrl[H];
-    int shift;
+    int shift;            // the shift of the row with the largest sum of |D|, less 3
+    unsigned long long rows;   // a row's shift beyond it, below 16: four bits each
 };
 
 // Parameters of the native kernel: EOS constants, c[k] = binom(gamma, k+1)

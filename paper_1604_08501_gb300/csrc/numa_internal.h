@@ -73,14 +73,14 @@ int gll_diff_matrix(int N, double *D);
 void sweep_tables(int N, const double *D, double De[16], double Do[16], double Dc[4],
                   double Dcr[4]);
 
-// The same tables as integers D 2^shift, cut into (high, low) words at bit
-// kFixLow (fixed_sweep.cuh): the arrays of a FixedTables; the shift is returned.
+// The same tables as integers, each row at its own scale, cut into (high, low) words
+// (fixed_sweep.cuh): the arrays of a FixedTables; its shift is returned.
 int fixed_tables(int N, const double *D, int *Deh, int *Del, int *Doh, int *Dol, int *Dch, int *Dcl,
-                 int *Dcrh, int *Dcrl);
+                 int *Dcrh, int *Dcrl, unsigned long long *rows);
 template <int T, int H>
 void fixed_tables(int N, const double *D, FixedTables<T, H> *f) {
     *f = FixedTables<T, H>{};
-    f->shift = fixed_tables(N, D, f->Deh, f->Del, f->Doh, f->Dol, f->Dch, f->Dcl, f->Dcrh, f->Dcrl);
+    f->shift = fixed_tables(N, D, f->Deh, f->Del, f->Doh, f->Dol, f->Dch, f->Dcl, f->Dcrh, f->Dcrl, &f->rows);
 }
 
 // Native: vol_rhs_fp64_kernel (N <= 7); NativeHigh: vol_rhs_high_kernel<Nq, double>

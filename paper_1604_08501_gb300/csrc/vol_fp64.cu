@@ -6,8 +6,8 @@
 // reference directions, the three D sweeps, the Jinv scaling and the gravity
 // source (Sec. 2, Eq. (2); sign and flux form of the paper's r/s subroutines,
 // Sec. 3).  State, geometry, pressure, fluxes and rhs are FP64; the D sweeps
-// run in 64-bit fixed point (fixed_sweep.cuh), whose error is below the FP64
-// sweeps'.
+// run in 64-bit fixed point (fixed_sweep.cuh: its bound, and its error beside the
+// FP64 sweep's).
 //
 // On GB300 the FP64 pipe (1.67 DFMA per clock and SM, 0.53 T/s) binds this
 // kernel, so the design minimises FP64 instructions per point:
@@ -22,21 +22,18 @@
 //    even-odd split of the GLL D (D[N-i][N-n] = -D[i][n]), half the multiplies
 //    of the direct sweep, on the integer pipes: no FP64 operation.  The sweeps
 //    and the sums over the directions were 100 of 157 FP64 operations per point
-//    at Nq = 8.  One thread's integers take 64 registers, as two CTAs of 512
-//    threads allow, and the integer work of one CTA runs beside the FP64 work
-//    of the other.  Measured at N = 7, 32768 elements: 4.949 ms with FP64
-//    sweeps, 1.881 ms (59 FP64 operations' time per point) in fixed point;
-//    N = 4, 512 elements, a call among others: 22.5 and 14.3 us.
+//    at Nq = 8.  The integer work of one CTA runs beside the FP64 work of the
+//    others on its SM.  Measured at N = 7, 32768 elements, with two CTAs of 512
+//    threads: 4.949 ms with FP64 sweeps, 1.881 ms (59 FP64 operations' time per
+//    point) in fixed point.
 //  * Jinv is applied once to the sum of the three sweeps (opt. level 8), as an
 //    integer multiply before the one rounding to FP64; the last terms of the
 //    pressure series are FP32 and 1/rho starts from an FP32 reciprocal
-//    (fp64_ops.cuh).  That leaves 47 of 59 FP64 operations per point: 3.5
-//    million points N = 3 383 -> 325 us, N = 4 397 -> 332 us, N = 5 394 -> 334 us;
-//    N = 7 needed smaller CTAs as well (vol_rhs_fp64_eight_kernel): 32768
-//    elements 1.881 -> 1.656 ms, the FP64 pipe 76 % busy of the 83 % that a loop of
-//    DFMAs reaches.  Later steps (fix_mad_wide; these sums in two groups of
-//    fields): N = 7 1.533 ms, N = 3 318 us, N = 4 330 us, 512 elements of N = 4
-//    12.3 us a call.
+//    (fp64_ops.cuh).  That leaves 47 of 59 FP64 operations per point; N = 7 needed
+//    smaller CTAs as well (vol_rhs_fp64_eight_kernel).  With these, fix_mad_wide
+//    and the sums in two groups of fields: N = 7 1.881 -> 1.535 ms, 3.5 million
+//    points of N = 3 383 -> 318 us, N = 4 397 -> 334 us, N = 5 394 -> 330 us, 512
+//    elements of N = 4 22.5 us with FP64 sweeps, 14.4 us so.
 //
 // One CTA of Nq^3 threads per element (several elements from Nq = 6 down, so
 // that a CTA has a few hundred threads: cta_elements), in three phases: fluxes by point,
@@ -107,7 +104,7 @@ __device__ __forceinline__ int dir_line(int d, int i, int j, int k) {
 template <int NQ, bool TRACERS>
 __global__ void __launch_bounds__((cta_threads<NQ>()), min_ctas<NQ>())
 vol_rhs_fp64_kernel(DeviceGeometry geo, const __grid_constant__ NativeParams P,
-                    FixedTables<16, 4> fix, const double *__restrict__ q,
+                    const __grid_constant__ FixedTables<16, 4> fix, const double *__restrict__ q,
                     double *__restrict__ rhs, int64_t M, int64_t e0, int64_t e_end, int nf_run) {
     constexpr int N3 = NQ * NQ * NQ;
     constexpr int NL = NQ * NQ;               // lines per (direction, field)
@@ -139,22 +136,25 @@ vol_rhs_fp64_kernel(DeviceGeometry geo, const __grid_constant__ NativeParams P,
 
     // ---- phase 2: even-odd sweeps, one line per task, in place --------
     for (int item = l; item < 3 * nf * EL; item += NT)   // a block's lines are contiguous
-        sE[item] = (short)sweep_line_fixed<NQ>(sF + (item / EL) * EW, item % EL, P, fix);
+        sweep_line_to<NQ>(sF + (item / EL) * EW, item % EL, P, fix, sE + item, 3 * nf * EL);
     __syncthreads();
     if (!active) return;
 
     // ---- phase 3: combine, scale, gravity, store ----------------------
     const double Jinv = geo.Jinv[node];
     const double drho = q[node] - geo.rho_ref[node];
-    int sl[3], ln[3];
+    int sl[3], ln[3], sh[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
+        const FixedRow row = fixed_row<NQ>(fix, d * nf * EL + el * NL + dir_line<NQ>(d, i, j, k),
+                                           d == 0 ? i : d == 1 ? j : k, 3 * nf * EL);
         sl[d] = d * nf * EW + el * N3 + dir_slot<NQ, double>(d, i, j, k);
-        ln[d] = d * nf * EL + el * NL + dir_line<NQ>(d, i, j, k);
+        ln[d] = row.at;
+        sh[d] = row.shift;
     }
     auto store = [&](auto &v, int b0) {   // fields b0 ..
         constexpr int NB = sizeof(v) / sizeof(double);
-        fixed_sums<NQ>(v, fix.shift, Jinv, [&](int d, int b) { return sF[sl[d] + (b0 + b) * EW]; },
+        fixed_sums<NQ>(v, sh, Jinv, [&](int d, int b) { return sF[sl[d] + (b0 + b) * EW]; },
                        [&](int d, int b) { return (int)sE[ln[d] + (b0 + b) * EL]; });
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
@@ -171,7 +171,7 @@ vol_rhs_fp64_kernel(DeviceGeometry geo, const __grid_constant__ NativeParams P,
         for (int b = kFields; b < kMaxFields; ++b) {
             if (b >= nf) break;
             double w[1];
-            fixed_sums<NQ>(w, fix.shift, Jinv, [&](int d, int) { return sF[sl[d] + b * EW]; },
+            fixed_sums<NQ>(w, sh, Jinv, [&](int d, int) { return sF[sl[d] + b * EW]; },
                            [&](int d, int) { return (int)sE[ln[d] + b * EL]; });
             rhs[b * M + node] = w[0];
         }
@@ -199,7 +199,7 @@ __device__ __forceinline__ constexpr int eight_block(int d, int b) { return d < 
 
 __global__ void __launch_bounds__(kEightThreads, 4)
 vol_rhs_fp64_eight_kernel(DeviceGeometry geo, const __grid_constant__ NativeParams P,
-                          FixedTables<16, 4> fix, const double *__restrict__ q, double *rhs,
+                          const __grid_constant__ FixedTables<16, 4> fix, const double *__restrict__ q, double *rhs,
                           int64_t M, int64_t e0) {
     constexpr int NQ = kEight, N3 = 512, NL = 64, NT = kEightThreads;
     extern __shared__ __align__(16) double sF[];                       // [block][slot]
@@ -225,7 +225,7 @@ vol_rhs_fp64_eight_kernel(DeviceGeometry geo, const __grid_constant__ NativePara
     // ---- phase 2: the sweeps of the 13 blocks, one line per task -----------
 #pragma unroll 1
     for (int item = l; item < kEightBlocks * NL; item += NT)
-        sE[item] = (short)sweep_line_fixed<NQ>(sF + (item / NL) * N3, item % NL, P, fix);
+        sweep_line_to<NQ>(sF + (item / NL) * N3, item % NL, P, fix, sE + item, 0);
     __syncthreads();
     // ---- phase 3: the momenta; the waiting fluxes into blocks 10 and 11, whose
     // slots of these points this thread alone has read
@@ -233,16 +233,18 @@ vol_rhs_fp64_eight_kernel(DeviceGeometry geo, const __grid_constant__ NativePara
     for (int x = 0; x < 2; ++x) {
         const int k = k0 + 4 * x;
         const int64_t node = node0 + x * NT;
-        int sl[3], ln[3];
+        int sl[3], ln[3], sh[3];
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
+            const FixedRow row = fixed_row<NQ>(fix, dir_line<NQ>(d, i, j, k), d == 0 ? i : d == 1 ? j : k, 0);
             sl[d] = dir_slot<NQ, double>(d, i, j, k);
-            ln[d] = dir_line<NQ>(d, i, j, k);
+            ln[d] = row.at;
+            sh[d] = row.shift;
         }
         const double f0 = rhs[node], f4 = rhs[4 * M + node];
         const double drho = q[node] - geo.rho_ref[node];
         double v[3];
-        fixed_sums<NQ>(v, fix.shift, geo.Jinv[node],
+        fixed_sums<NQ>(v, sh, geo.Jinv[node],
                        [&](int d, int b) { return sF[eight_block(d, b + 1) * N3 + sl[d]]; },
                        [&](int d, int b) { return (int)sE[eight_block(d, b + 1) * NL + ln[d]]; });
         rhs[M + node] = v[0];
@@ -253,21 +255,23 @@ vol_rhs_fp64_eight_kernel(DeviceGeometry geo, const __grid_constant__ NativePara
     }
     __syncthreads();
     if (l < 2 * NL)
-        sE[10 * NL + l] = (short)sweep_line_fixed<NQ>(sF + (10 + l / NL) * N3, l % NL, P, fix);
+        sweep_line_to<NQ>(sF + (10 + l / NL) * N3, l % NL, P, fix, sE + 10 * NL + l, 0);
     __syncthreads();
     // ---- rho and Theta
 #pragma unroll 1
     for (int x = 0; x < 2; ++x) {
         const int k = k0 + 4 * x;
         const int64_t node = node0 + x * NT;
-        int sl[3], ln[3];
+        int sl[3], ln[3], sh[3];
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
+            const FixedRow row = fixed_row<NQ>(fix, dir_line<NQ>(d, i, j, k), d == 0 ? i : d == 1 ? j : k, 0);
             sl[d] = dir_slot<NQ, double>(d, i, j, k);
-            ln[d] = dir_line<NQ>(d, i, j, k);
+            ln[d] = row.at;
+            sh[d] = row.shift;
         }
         double v[2];
-        fixed_sums<NQ>(v, fix.shift, geo.Jinv[node],
+        fixed_sums<NQ>(v, sh, geo.Jinv[node],
                        [&](int d, int b) { return sF[(d < 2 ? 5 * d + 4 * b : 10 + b) * N3 + sl[d]]; },
                        [&](int d, int b) { return (int)sE[(d < 2 ? 5 * d + 4 * b : 10 + b) * NL + ln[d]]; });
         rhs[node] = v[0];
@@ -279,7 +283,8 @@ template <int NQ, bool TRACERS>
 cudaError_t launch_kernel(ElemRange r, int nf, const DeviceGeometry &geo, const NativeParams &P,
                           const FixedTables<16, 4> &fix, const double *q, double *rhs, cudaStream_t s) {
     constexpr int EPC = cta_elements<NQ>(), NT = cta_threads<NQ>();
-    const size_t smem = (sizeof(double) * NQ + sizeof(short)) * EPC * NQ * NQ * nf * 3;
+    const size_t smem =
+        (sizeof(double) * NQ + sizeof(short) * line_exponents<NQ>()) * EPC * NQ * NQ * nf * 3;
     // The opt-in above 48 KB is per device; setting it on every launch keeps
     // multi-device processes correct and costs about a microsecond.
     cudaError_t e = cudaFuncSetAttribute(vol_rhs_fp64_kernel<NQ, TRACERS>,

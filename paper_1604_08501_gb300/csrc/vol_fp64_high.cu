@@ -149,7 +149,7 @@ template <int NQ, typename T, int NF>
 __host__ __device__ constexpr size_t high_smem_bytes() {
     return sizeof(T) * ((sizeof(T) == 8 ? 4 * NQ * NQ * NQ : 0) +
                         high_group<NQ, T, NF>() * 3 * NQ * NQ * line_stride<NQ, T>()) +
-           (sizeof(T) == 8 ? sizeof(short) * high_group<NQ, T, NF>() * 3 * NQ * NQ : 0);
+           (sizeof(T) == 8 ? sizeof(short) * line_exponents<NQ>() * high_group<NQ, T, NF>() * 3 * NQ * NQ : 0);
 }
 
 // CTAs per SM the register budget is sized for: two where two CTAs' shared
@@ -419,8 +419,8 @@ vol_rhs_high_kernel(typename HighTypes<T>::Geo geo,
                     if constexpr (MIXED)
                         sweep_line<NQ>(sF + (gl * 3 + slab) * FB, c, P);
                     else
-                        sE[(gl * 3 + slab) * NL + c] =
-                            (short)sweep_line_fixed<NQ>(sF + (gl * 3 + slab) * FB, c, P, P.fix);
+                        sweep_line_to<NQ>(sF + (gl * 3 + slab) * FB, c, P, P.fix,
+                                          sE + (gl * 3 + slab) * NL + c, G * 3 * NL);
                 }
             }
         } else {
@@ -466,14 +466,15 @@ vol_rhs_high_kernel(typename HighTypes<T>::Geo geo,
                         v = -jinv * (F[s0] + F[FB + s1] + F[2 * FB + s2]);
                     } else {
                         const short *E = sE + gl * 3 * NL;
+                        const FixedRow r0 = fixed_row<NQ>(P.fix, NQ * k + j, i, G * 3 * NL),
+                                       r1 = fixed_row<NQ>(P.fix, NL + NQ * k + i, j, G * 3 * NL),
+                                       r2 = fixed_row<NQ>(P.fix, 2 * NL + NQ * j + i, k, G * 3 * NL);
+                        const int sh[3] = {r0.shift, r1.shift, r2.shift};
                         T w[1];
                         fixed_sums<NQ>(
-                            w, P.fix.shift, jinv,
+                            w, sh, jinv,
                             [&](int d, int) { return F[d == 0 ? s0 : d == 1 ? FB + s1 : 2 * FB + s2]; },
-                            [&](int d, int) {
-                                return (int)E[d == 0 ? NQ * k + j : d == 1 ? NL + NQ * k + i
-                                                                           : 2 * NL + NQ * j + i];
-                            });
+                            [&](int d, int) { return (int)E[d == 0 ? r0.at : d == 1 ? r1.at : r2.at]; });
                         v = w[0];
                     }
                     if (b == 3) {

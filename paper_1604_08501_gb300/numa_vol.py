@@ -54,8 +54,8 @@ def diff_matrix(N: int) -> np.ndarray:
 class VolumeTerm:
     """One mesh on the current CUDA device (numa_vol_create ... numa_vol_destroy).
 
-    precision: "fp64" (FP64 arithmetic, the D sums no less exact), "df64" (double-float
-    arithmetic on the FP32 pipes, N = 7) or "mixed" (FP32 perturbation state,
+    precision: "fp64" (FP64 arithmetic, the D sums in 64-bit fixed point), "df64" (double-float
+    arithmetic on the FP32 pipes, N <= 7) or "mixed" (FP32 perturbation state,
     see workload.perturbation_state)."""
 
     def __init__(self, N: int, num_elements: int, g, Jinv, rho_ref, rhotheta_ref,
