@@ -328,14 +328,16 @@ int numa_batch_advance(numa_batch *b, int nsteps, double dt, void *stream);
  * keeping a change that saves at least 1 %. */
 int numa_batch_autotune(numa_batch *b, void *stream);
 
-/* Launch configuration of a batch.  Indices are Nq = N + 1 (2..8; 0 and 1
- * unused). */
+/* Launch configuration of a batch.  Indices are Nq = N + 1 (2..8; 1 unused). */
 typedef struct {
     int tile[9];               /* elements per work item: a positive multiple of
                                   512 / Nq^3 (the elements one pass of 512
-                                  threads holds).  The default, four passes, is
-                                  split finer in launches of few items until it
-                                  is set or autotuned */
+                                  threads holds).  Tiles that are set or
+                                  autotuned run as they are; the default, four
+                                  passes, is split finer in launches of few
+                                  items.  tile[0]: 1 while the tiles are that
+                                  default, else 0; set_config with 1 there and
+                                  four passes everywhere goes back to it */
     int sweep[9];              /* NUMA_SWEEP_CUDA_CORES or NUMA_SWEEP_TENSOR_TF32 */
     int ctas_per_sm;           /* CTAs per SM of the persistent grid: 1 .. 2
                                   (NUMA_MIXED); NUMA_FP64 has one grid (two CTAs
@@ -361,7 +363,7 @@ int numa_batch_get_config(const numa_batch *b, numa_batch_config *out);
  * NUMA_FP64 batch). */
 int numa_batch_set_config(numa_batch *b, const numa_batch_config *c);
 
-/* Elements per work item the batch uses for order Nq (2..8). */
+/* Elements per work item of order Nq (2..8): the configuration's tile. */
 int numa_batch_tile(const numa_batch *b, int nq);
 
 /*

@@ -48,16 +48,20 @@ bool has_tracers(const std::vector<numa::BatchInstance> &v) {
 
 }  // namespace
 
+namespace numa {
+constexpr int kDefaultPasses = 4;   // per work item
+}
+
 struct numa_batch {
     numa_precision prec = NUMA_FP64;
     int device = 0;
     int num_sms = 0;
     std::vector<numa::BatchInstance> inst;
-    int tile_mult[9] = {4, 4, 4, 4, 4, 4, 4, 4, 4};   // elements per item / elements per pass, by Nq
+    int tile_mult[9];      // elements per item / elements per pass, by Nq
     numa_sweep sweep = NUMA_SWEEP_CUDA_CORES;
     unsigned tc_mask = 0;  // orders (bit Nq) whose D sums run on the tensor cores (mixed only)
     int ctas_per_sm = 0;   // CTAs per SM of the persistent grid (0: the kernel's maximum)
-    bool tile_chosen = false;       // by the autotuner or set_config; else at most these
+    bool tile_chosen = false;       // tiles set or tuned; else these are the most (fit_passes)
     bool costliest_first = false;   // work items sorted by points, largest first
     bool tmem_state = false;        // mixed, CUDA-core tiles: the state in tensor memory
     double tuned_ms = 0.0;          // last autotune: ms per step of the chosen configuration
@@ -184,6 +188,7 @@ int numa_batch_create(numa_precision prec, numa_batch **out) {
     numa_batch *b = new (std::nothrow) numa_batch();
     if (!b) return bfail(NUMA_ENOMEM, "numa_batch_create: host allocation failed");
     b->prec = prec;
+    std::fill(b->tile_mult, b->tile_mult + 9, numa::kDefaultPasses);
     b->tmem_state = prec == NUMA_MIXED;   // the state in tensor memory: the faster tile
     cudaError_t e = cudaGetDevice(&b->device);
     if (e == cudaSuccess)
@@ -460,7 +465,8 @@ int numa_batch_get_config(const numa_batch *b, numa_batch_config *out) {
     if (!b || !out) return bfail(NUMA_EINVAL, "numa_batch_get_config: NULL argument");
     numa_batch_config c{};
     for (int nq = 0; nq < 9; ++nq) {
-        c.tile[nq] = nq >= 2 ? numa::elements_per_pass(nq) * b->tile_mult[nq] : 0;
+        c.tile[nq] = nq >= 2 ? numa::elements_per_pass(nq) * b->tile_mult[nq]
+                             : (nq == 0 && !b->tile_chosen ? 1 : 0);
         c.sweep[nq] = ((b->tc_mask >> nq) & 1u) ? NUMA_SWEEP_TENSOR_TF32 : NUMA_SWEEP_CUDA_CORES;
     }
     c.ctas_per_sm = b->ctas_per_sm;
@@ -495,8 +501,11 @@ int numa_batch_set_config(numa_batch *b, const numa_batch_config *c) {
             return bfail(NUMA_EINVAL, "numa_batch_set_config: a sweep is not CUDA_CORES or TENSOR_TF32");
         }
     }
+    // tiles given run as given, also where they equal the default; tile[0], as
+    // get_config reports it for tiles never set, keeps the default automatic
+    b->tile_chosen = c->tile[0] == 0;
     for (int nq = 2; nq <= 8; ++nq) {
-        b->tile_chosen = b->tile_chosen || b->tile_mult[nq] != mult[nq];
+        b->tile_chosen = b->tile_chosen || mult[nq] != numa::kDefaultPasses;
         b->tile_mult[nq] = mult[nq];
     }
     b->tc_mask = mask;

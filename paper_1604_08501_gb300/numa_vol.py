@@ -244,9 +244,12 @@ class Batch:
 
     def set_config(self, tile=None, sweep=None, ctas_per_sm=None, costliest_first=None,
                    state_in_tmem=None) -> None:
-        """Set any of the configuration fields of config() (the others stay)."""
+        """Set any of the configuration fields of config() (the others stay).  Tiles that
+        are given run as they are; the default ones are split finer in small launches."""
         cur = self.config()
         c = _lib.numa_batch_config()
+        if not tile:   # tiles never set stay automatic (the configuration's tile[0])
+            check_batch(_lib.load().numa_batch_get_config(self.handle, C.byref(c)))
         for nq in range(2, 9):
             c.tile[nq] = int((tile or {}).get(nq, cur["tile"][nq]))
             c.sweep[nq] = self.SWEEPS[(sweep or {}).get(nq, cur["sweep"][nq])]
