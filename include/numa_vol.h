@@ -221,9 +221,10 @@ void numa_vol_destroy(numa_vol *h);
 
 /* Name of the kernel numa_vol_rhs launches for this handle:
  * "vol_rhs_fp64_kernel<Nq>" (NUMA_FP64, or NUMA_DF64 after a geometry
- * fallback), "vol_rhs_df64_kernel<Nq>", "vol_rhs_mixed_kernel<Nq>" or
- * "vol_rhs_high_kernel<Nq, type>" (the kernel's name without the forms that a
- * launch's size chooses among).  Static string; "" for a NULL handle. */
+ * fallback), "vol_rhs_df64_kernel<Nq>", "vol_rhs_mixed_kernel<Nq>",
+ * "vol_rhs_mixed_tc_kernel<8>" or "vol_rhs_high_kernel<Nq, type>": the function's
+ * name and leading template arguments, which every form has that a launch's
+ * size and field count choose among.  Static string; "" for a NULL handle. */
 const char *numa_vol_kernel_name(const numa_vol *h);
 
 /*

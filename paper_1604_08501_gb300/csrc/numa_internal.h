@@ -84,8 +84,8 @@ void fixed_tables(int N, const double *D, FixedTables<T, H> *f) {
 }
 
 // Native: vol_rhs_fp64_kernel (N <= 7); NativeHigh: vol_rhs_high_kernel<Nq, double>
-// (N = 8..15); DoubleFloat (vol_rhs_df64_kernel<Nq>, N <= 7); Mixed (N <= 7) and MixedHigh:
-// vol_rhs_high_kernel<Nq, float> (N = 8..15).
+// (N = 8..15); DoubleFloat: vol_rhs_df64_kernel (N <= 7); Mixed: vol_rhs_mixed_kernel
+// (N <= 7); MixedHigh: vol_rhs_high_kernel<Nq, float> (N = 8..15, both forms).
 enum class Kernel { Native, NativeHigh, DoubleFloat, Mixed, MixedHigh };
 
 // Device-side description of one instance of a batch: its order, size, state

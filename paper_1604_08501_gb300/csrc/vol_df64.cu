@@ -411,7 +411,7 @@ vol_rhs_df64_kernel(DfGeometry geo, const __grid_constant__ DfParams P, const do
 
 // N = 7 without tracers: 256 threads per element, two points each, four CTAs per
 // SM instead of two of 512 threads, and 13 of the 15 flux blocks in shared
-// memory, as in vol_rhs_fp64_eight_kernel (vol_fp64.cu): the t fluxes of rho and
+// memory, as in vol_rhs_fp64_kernel<8, TwoPoints> (vol_fp64.cu): the t fluxes of rho and
 // Theta wait in their outputs' places of rhs until the momenta are done.  The
 // operations are those of vol_rhs_df64_kernel<8>, so the results are the same bit
 // for bit; that kernel takes the launches of fewer than three elements per SM,
@@ -422,11 +422,14 @@ constexpr int kEightThreads = 256, kEightBlocks = 13;
 constexpr size_t kEightSmem = kEightBlocks * sizeof(float2) * 512;
 __device__ __forceinline__ constexpr int eight_block(int d, int b) { return d < 2 ? 5 * d + b : 9 + b; }
 
+struct TwoPoints {};   // the form's name: vol_rhs_df64_kernel<8, TwoPoints>
+template <int NQ, typename Form>
 __global__ void __launch_bounds__(kEightThreads, 4)
-vol_rhs_df64_eight_kernel(DfGeometry geo, const __grid_constant__ DfParams P,
+vol_rhs_df64_kernel(DfGeometry geo, const __grid_constant__ DfParams P,
                           const double *__restrict__ q, double *rhs, int64_t M, int64_t e0,
                           int64_t e_end, int64_t ahead) {
-    constexpr int NQ = 8, N3 = 512, NL = 64, NT = kEightThreads;
+    static_assert(NQ == 8, "two points a thread: 512 points");
+    constexpr int N3 = 512, NL = 64, NT = kEightThreads;
     extern __shared__ float2 sbuf[];   // [block][slot]
     const int l = threadIdx.x;
     const int i = l % NQ, j = (l / NQ) % NQ, k0 = l / NL;   // points (i, j, k0) and (i, j, k0 + 4)
@@ -569,12 +572,12 @@ cudaError_t launch_df(ElemRange r, int nf, const DfGeometry &geo, const DfParams
     if (nf > kFields) return launch_df_form<NQ, true>(r, nf, geo, P, q, rhs, num_sms, s);
     if constexpr (NQ == 8) {
         if (r.count >= 3 * (int64_t)num_sms) {
-            const cudaError_t e = cudaFuncSetAttribute(vol_rhs_df64_eight_kernel,
+            const cudaError_t e = cudaFuncSetAttribute(vol_rhs_df64_kernel<8, TwoPoints>,
                                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                        (int)kEightSmem);
             if (e != cudaSuccess) return e;
             const int64_t ahead = num_sms > 0 ? 2 * (int64_t)num_sms : 1;   // half a wave
-            vol_rhs_df64_eight_kernel<<<(unsigned)r.count, kEightThreads, kEightSmem, s>>>(
+            vol_rhs_df64_kernel<8, TwoPoints><<<(unsigned)r.count, kEightThreads, kEightSmem, s>>>(
                 geo, P, q, rhs, r.M, r.e0, r.e0 + r.count, ahead);
             return cudaGetLastError();
         }

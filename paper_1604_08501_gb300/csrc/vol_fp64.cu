@@ -30,7 +30,7 @@
 //    integer multiply before the one rounding to FP64; the last terms of the
 //    pressure series are FP32 and 1/rho starts from an FP32 reciprocal
 //    (fp64_ops.cuh).  That leaves 47 of 59 FP64 operations per point; N = 7 needed
-//    smaller CTAs as well (vol_rhs_fp64_eight_kernel).  With these, fix_mad_wide
+//    smaller CTAs as well (vol_rhs_fp64_kernel<8, TwoPoints>).  With these, fix_mad_wide
 //    and the sums in two groups of fields: N = 7 1.881 -> 1.535 ms, 3.5 million
 //    points of N = 3 383 -> 318 us, N = 4 397 -> 334 us, N = 5 394 -> 330 us, 512
 //    elements of N = 4 22.5 us with FP64 sweeps, 14.4 us so.
@@ -197,11 +197,14 @@ constexpr size_t kEightSmem = kEightBlocks * (sizeof(double) * 512 + sizeof(shor
 // Block of direction d and field b: 5 d + b for r and s; t: the momenta's 10, 11, 12.
 __device__ __forceinline__ constexpr int eight_block(int d, int b) { return d < 2 ? 5 * d + b : 9 + b; }
 
+struct TwoPoints {};   // the form's name: vol_rhs_fp64_kernel<8, TwoPoints>
+template <int NQ, typename Form>
 __global__ void __launch_bounds__(kEightThreads, 4)
-vol_rhs_fp64_eight_kernel(DeviceGeometry geo, const __grid_constant__ NativeParams P,
+vol_rhs_fp64_kernel(DeviceGeometry geo, const __grid_constant__ NativeParams P,
                           const __grid_constant__ FixedTables<16, 4> fix, const double *__restrict__ q, double *rhs,
                           int64_t M, int64_t e0) {
-    constexpr int NQ = kEight, N3 = 512, NL = 64, NT = kEightThreads;
+    static_assert(NQ == kEight, "two points a thread: 512 points");
+    constexpr int N3 = 512, NL = 64, NT = kEightThreads;
     extern __shared__ __align__(16) double sF[];                       // [block][slot]
     short *sE = reinterpret_cast<short *>(sF + kEightBlocks * N3);     // [block][line]
     const int l = threadIdx.x;
@@ -302,11 +305,11 @@ cudaError_t launch_nq(ElemRange r, int nf, const DeviceGeometry &geo, const Nati
     if (nf == kFields) {
         if constexpr (NQ == kEight) {
             if (r.count >= 6 * (int64_t)num_sms) {
-                const cudaError_t e = cudaFuncSetAttribute(vol_rhs_fp64_eight_kernel,
+                const cudaError_t e = cudaFuncSetAttribute(vol_rhs_fp64_kernel<kEight, TwoPoints>,
                                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                            (int)kEightSmem);
                 if (e != cudaSuccess) return e;
-                vol_rhs_fp64_eight_kernel<<<(unsigned)r.count, kEightThreads, kEightSmem, s>>>(
+                vol_rhs_fp64_kernel<kEight, TwoPoints><<<(unsigned)r.count, kEightThreads, kEightSmem, s>>>(
                     geo, P, fix, q, rhs, r.M, r.e0);
                 return cudaGetLastError();
             }

@@ -79,7 +79,8 @@ struct PointLoads {
     float q[NF], g[9], rho_ref, theta_ref;
 };
 
-template <int NQ, int NF>
+struct Planes {};   // the form's name: vol_rhs_high_kernel<Nq, float, NF, Planes>
+template <int NQ, typename T, int NF, typename Form>
 __global__ void __launch_bounds__((Plane<NQ, NF>::NT), (Plane<NQ, NF>::CTAS))
 vol_rhs_high_kernel(MixedGeometry geo, HighParams32 P, const float *__restrict__ q, float *rhs,
                     int64_t M, int64_t e0, int nf, int64_t e_end, int64_t ahead) {
@@ -277,11 +278,11 @@ template <int NQ, int NF>
 cudaError_t launch_plane(ElemRange r, int nf, const MixedGeometry &geo, const HighParams32 &P,
                          const float *q, float *rhs, int num_sms, cudaStream_t s) {
     using S = Plane<NQ, NF>;
-    const cudaError_t e = cudaFuncSetAttribute(vol_rhs_high_kernel<NQ, NF>,
+    const cudaError_t e = cudaFuncSetAttribute(vol_rhs_high_kernel<NQ, float, NF, Planes>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
     if (e != cudaSuccess) return e;
     const int64_t ahead = (int64_t)num_sms * S::CTAS;   // one wave
-    vol_rhs_high_kernel<NQ, NF><<<(unsigned)r.count, S::NT, S::SMEM, s>>>(
+    vol_rhs_high_kernel<NQ, float, NF, Planes><<<(unsigned)r.count, S::NT, S::SMEM, s>>>(
         geo, P, q, rhs, r.M, r.e0, nf, r.e0 + r.count, ahead);
     return cudaGetLastError();
 }
