@@ -414,7 +414,8 @@ def roofline_entries(kname, kernel_ms, w):
     if "mixed" in kname:
         return hbm, None
     native = kname.startswith("vol_rhs_fp64")
-    flops = FP64_PIPE_FLOPS_NATIVE if native else flops_per_node_fp64(w.N + 1)
+    # N = 1 sweeps in FP64: the operation's own count stands for it
+    flops = FP64_PIPE_FLOPS_NATIVE if native and w.N >= 2 else flops_per_node_fp64(w.N + 1)
     fp64_tfs = flops * w.M / (kernel_ms * 1e-3) / 1e12
     # FP64 flop rate (the native kernel: what it issues on the FP64 pipe; the
     # double-float kernel: the FP64 operation's equivalent) against the FP64 pipe of one GB300 (152 SMs x
