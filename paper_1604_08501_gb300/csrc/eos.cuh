@@ -88,8 +88,8 @@ static __device__ __forceinline__ double pressure_perturbation(double Th, double
 }
 
 // FP32 form from the perturbation Theta' itself (mixed precision): the series
-// (5 or 16 terms) or expm1f(gamma log1pf(x)), chosen per warp as in FP64, all
-// free of cancellation.
+// (5 or 16 terms) or expm1f(gamma log1pf(x)), chosen per warp as in FP64 (N = 8..15:
+// per point), all free of cancellation.
 // A = K Theta_ref^(gamma - 1) with K = p0^(1 - gamma) R^gamma is recomputed
 // from Theta_ref instead of being read from memory.  eos_reference_f32 forms
 // the per-point factors (w = 1/Theta_ref and A), which a caller that keeps a
@@ -103,27 +103,37 @@ static __device__ __forceinline__ EosRef32 eos_reference_f32(float th0, const Pa
     return EosRef32{__frcp_rn(th0), P.K * exp2f(P.gm1 * log2f(th0))};   // A = p(Theta_ref)/Theta_ref
 }
 
-// Params: MixedParams or HighParams32 (c, K, gm1, gamma).
+// p' by the first TERMS terms of the series, sum_k c_{k+1} x^k.
+template <int TERMS, typename Params>
+static __device__ __forceinline__ float eos_series_f32(float thp, float x, float A, const Params &P) {
+    float g = P.c[TERMS - 1];
+#pragma unroll
+    for (int k = TERMS - 2; k >= 0; --k) g = fmaf(g, x, P.c[k]);
+    return (A * thp) * g;
+}
+
+// Params: MixedParams or HighParams32 (c, K, gm1, gamma).  GROUP = 1: each point its
+// own form, for the kernels of N = 8..15, which share an element out to warps in
+// two ways and give it the same result (a warp whose points all take the short
+// series still runs nothing else; without that N = 15 took 108.4 us instead of 103.3).
 template <int GROUP = 32, typename Params>
 static __device__ __forceinline__ float pressure_perturbation_f32(float thp, float th0, EosRef32 r,
                                                            const Params &P) {
-    const unsigned lanes = vote_mask<GROUP>();
+    const unsigned lanes = vote_mask<GROUP == 1 ? 32 : GROUP>();
     if (__all_sync(lanes, th0 > 0.0f)) {
         const float x = thp * r.w;
         const float ax = fabsf(x);
-        if (__all_sync(lanes, ax <= 0.015625f)) {
-            float g = P.c[4];
-#pragma unroll
-            for (int k = 3; k >= 0; --k) g = fmaf(g, x, P.c[k]);   // sum_k c_{k+1} x^k
-            return (r.A * thp) * g;
+        if (__all_sync(lanes, ax <= 0.015625f)) return eos_series_f32<5>(thp, x, r.A, P);
+        if constexpr (GROUP > 1) {
+            if (__all_sync(lanes, ax <= 0.5f)) return eos_series_f32<16>(thp, x, r.A, P);
+            if (__all_sync(lanes, x > -1.0f)) return (r.A * th0) * expm1f(P.gamma * log1pf(x));
         }
-        if (__all_sync(lanes, ax <= 0.5f)) {
-            float g = P.c[15];
-#pragma unroll
-            for (int k = 14; k >= 0; --k) g = fmaf(g, x, P.c[k]);
-            return (r.A * thp) * g;
-        }
-        if (__all_sync(lanes, x > -1.0f)) return (r.A * th0) * expm1f(P.gamma * log1pf(x));
+    }
+    if constexpr (GROUP == 1) {
+        const float x = thp * r.w;
+        const float ax = fabsf(x);
+        if (th0 > 0.0f && ax <= 0.015625f) return eos_series_f32<5>(thp, x, r.A, P);
+        if (th0 > 0.0f && ax <= 0.5f) return eos_series_f32<16>(thp, x, r.A, P);
     }
     // Theta_ref = 0 (the paper's full-pressure form): p' = p(Theta'); and,
     // per lane, whatever the warp's common forms do not cover.

@@ -283,7 +283,7 @@ vol_rhs_high_kernel(typename HighTypes<T>::Geo geo,
                 T rinv, pp, Th;
                 if constexpr (MIXED) {
                     const float th0 = geo.theta_ref[node];
-                    pp = pressure_perturbation_f32(q[4 * M + node], th0, P);
+                    pp = pressure_perturbation_f32<1>(q[4 * M + node], th0, P);
                     rinv = __frcp_rn(geo.rho_ref[node] + q[node]);
                     Th = th0 + q[4 * M + node];
                 } else {

@@ -145,7 +145,7 @@ vol_rhs_high_kernel(MixedGeometry geo, HighParams32 P, const float *__restrict__
                 const PointLoads<NF> &x = pt[p];
                 const float U[3] = {x.q[1], x.q[2], x.q[3]};
                 const float Th = x.theta_ref + x.q[4];
-                const float pp = pressure_perturbation_f32(x.q[4], x.theta_ref, P);
+                const float pp = pressure_perturbation_f32<1>(x.q[4], x.theta_ref, P);
                 const float rinv = __frcp_rn(x.rho_ref + x.q[0]);
 #pragma unroll
                 for (int d = 0; d < 3; ++d) {
@@ -292,7 +292,8 @@ cudaError_t launch_plane(ElemRange r, int nf, const MixedGeometry &geo, const Hi
 // element and planes: 4 elements of N = 8 9.1 and 10.6, N = 14 14.5 and 20.5; 150
 // elements of N = 8 9.5 and 12.4, N = 14 24.0 and 26.2; 504 elements of N = 8 18.1
 // and 17.4, N = 14 81.9 and 57.4).  The line is drawn by the mesh, not by the
-// launch, so that a chunk of the host path computes what the whole mesh does.
+// launch; both kernels give an element the same bits
+// (tests/test_gpu_high_mesh_size.py).
 template <int NQ>
 cudaError_t launch_nq(ElemRange r, int nf, const MixedGeometry &geo, const HighParams32 &P,
                       const float *q, float *rhs, int num_sms, cudaStream_t s) {
