@@ -140,8 +140,10 @@ typedef struct numa_vol numa_vol;
  *
  * NUMA_FP64 and NUMA_DF64 compute the same operation.  Both evaluate
  * p(Theta) - p(Theta_ref) as p_ref ((1 + x)^gamma - 1) in x =
- * (Theta - Theta_ref)/Theta_ref: NUMA_FP64 by its binomial series (|x| <= 1/8)
- * or expm1(gamma log1p(x)), the form chosen per warp of 32 points;
+ * (Theta - Theta_ref)/Theta_ref: NUMA_FP64 by its binomial series (|x| <= 1/8;
+ * for |x| <= 1/64 its last four terms, below 2^-34 of the sum, in FP32) or
+ * expm1(gamma log1p(x)), the form chosen per warp of 32 points, and 1/rho to
+ * 0.5005 units in the last place;
  * NUMA_DF64 by the series where |x| <= 1/64 and by pow elsewhere.  The error
  * of NUMA_FP64 against an exact evaluation is a few units of 2^-53 times the
  * condition number of the D sweeps (the ratio of
