@@ -126,8 +126,9 @@ typedef struct numa_vol numa_vol;
  * c->cp > c->R > 0 and c->p0 > 0.  On success *out receives the handle
  * (release with numa_vol_destroy).  Errors: NUMA_EINVAL, NUMA_ENOMEM,
  * NUMA_ECUDA, NUMA_EUNSUPPORTED (NUMA_DF64 with N > 7).
- * Handles of N > 7 evaluate one element per CTA of 3 or 4 (N+1)^2 threads,
- * the fields in groups (vol_rhs_high_kernel); the batch, the engine and
+ * Handles of N > 7 evaluate one element per CTA (vol_rhs_high_kernel): of 3 or 4
+ * (N+1)^2 threads, the fields in groups, or in NUMA_MIXED on larger meshes of
+ * (N+1)^2 threads that walk the k-planes; the batch, the engine and
  * numa_batch_advance_noalloc take handles of N <= 7.
  *
  * NUMA_MIXED takes the state as FP32 perturbations from the reference state:
@@ -181,14 +182,13 @@ int numa_vol_rhs(numa_vol *h, const void *q, void *rhs, void *stream);
 /*
  * Evaluate the volume term from HOST memory: copies q to the device, runs the
  * kernel, copies rhs back and waits for completion.  The mesh is processed in
- * 4 to 64 chunks of elements (about 10 MB of state each) on four
- * internal streams, so the copy-in of one
- * chunk, the kernel on the previous one and the copy-out of the one before
- * overlap; each chunk moves with one 2D copy per direction over all planes.  Device staging buffers
- * (2 x (5 + num_tracers) x M values) are allocated on the first call and
- * owned by the handle.  q and rhs are host pointers to 5 (+ num_tracers)
- * planes of M values of the
- * handle's state type (pinned memory gives full copy bandwidth).  Errors:
+ * chunks of elements (about 10 MB of state each; 4 to 64 of them, at most one
+ * per element) on four internal streams, so the copy-in of one chunk, the
+ * kernel on the previous one and the copy-out of the one before overlap; each
+ * chunk moves with one 2D copy per direction over all planes.  Device staging
+ * buffers (2 x (5 + num_tracers) x M values) are allocated on the first call
+ * and owned by the handle.  q and rhs are host pointers to 5 (+ num_tracers)
+ * planes of M values of the handle's state type (pinned memory gives full copy bandwidth).  Errors:
  * NUMA_EINVAL, NUMA_ENOMEM, NUMA_ECUDA.
  */
 int numa_vol_rhs_host(numa_vol *h, const void *q, void *rhs);

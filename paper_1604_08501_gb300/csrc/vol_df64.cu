@@ -58,8 +58,9 @@ struct DfShape {
     static constexpr int kItems = kFields * 3 * NL;    // (direction, field, line) sweep tasks
 };
 
-// Resident CTAs per SM the register budget is sized for: about 1024 threads at
-// every order (56 to 72 registers, up to 100 bytes spilled), at most 32 CTAs.
+// Resident CTAs per SM the register budget is sized for: about 1024 threads (56 to
+// 72 registers, up to 100 bytes spilled), at most 32 CTAs, so 256 and 864 threads
+// at Nq = 2 and 3, whose CTAs are one element of 8 and 27 threads.
 // The spills cost less than the warps they buy: 3.5 million points, us, at 640,
 // 704, 864 and 1029 threads per SM (Nq = 7: one, two, two and three CTAs):
 // Nq = 3 471 432 412 412, 4 198 185 178 178, 5 251 250 229 199, 6 321 235 207

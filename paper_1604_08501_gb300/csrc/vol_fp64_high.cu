@@ -26,8 +26,8 @@
 //    pass each CTA prefetches the element of the next wave to L2.
 // The FP64 D sweeps run in 64-bit fixed point on the integer pipes
 // (fixed_sweep.cuh), as at the low orders: measured on 3.5 million points, five
-// fields, N = 11 1.405 -> 0.685 ms, N = 15 1.569 -> 0.839 ms, with three tracers
-// 2.100 -> 0.951 and 2.365 -> 1.200 ms; what is left is bound by the latency of
+// fields, N = 11 1.405 -> 0.552 ms, N = 15 1.569 -> 0.693 ms, with three tracers
+// 2.100 -> 0.771 and 2.365 -> 0.978 ms; what is left is bound by the latency of
 // the passes' loads and barriers (a field at a time), no longer by the FP64 pipe.
 // (Meshes of two elements per SM and more run the mixed mode in
 // vol_mixed_high.cu where that is faster; a few elements finish sooner here, with
@@ -507,7 +507,11 @@ cudaError_t launch_high_form(ElemRange r, int nf, const Geo &geo, const Params &
     cudaError_t e = cudaFuncSetAttribute(vol_rhs_high_kernel<NQ, T, NF>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    int64_t ahead = 0;   // FP64: no prefetch (not measured since the sweeps left the FP64 pipe)
+    // FP64: no prefetch.  With the next wave's element prefetched as in FP32 (odd Nq
+    // rounded to 16-byte units), 3.5 million points, us, without and with: N = 8 606 592,
+    // 9 652 659, 10 615 633, 11 552 570, 12 825 776, 13 747 760, 14 710 724, 15 693
+    // 726; three tracers N = 11 771 795, 15 978 1023.
+    int64_t ahead = 0;
     if (sizeof(T) == 4 && num_sms > 0) {
         int per_sm = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, vol_rhs_high_kernel<NQ, T, NF>,

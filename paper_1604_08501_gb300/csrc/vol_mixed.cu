@@ -1,5 +1,6 @@
 // Mixed-precision element volume term (NUMA_MIXED), orders N = 1..7 (N = 8..15:
-// vol_fp64_high.cu), with or without passive tracers.
+// vol_mixed_high.cu, and vol_fp64_high.cu for small meshes and some forms), with or
+// without passive tracers.
 //
 // The operation of Sec. 2, Eq. (2) (sign and flux form of the paper's r/s
 // subroutines, Sec. 3) on FP32 data:
